@@ -122,7 +122,9 @@ int hp_plan_destroy(hp_plan* plan);
 #define HP_PARAM_W_TOL 4          /* merge: max |width index difference| (>= 0) */
 #define HP_PARAM_RAW_CAPACITY 5   /* raw-candidate scratch capacity (>= 1024) */
 #define HP_PARAM_DEDISP_CONFIG 6  /* dedispersion tile shape index (0..HP_NUM_DEDISP_CONFIGS-1), default 17;
-                                     12 while HP_PARAM_SUBBAND_CHANS > 0 unless a shape was set */
+                                     12 while HP_PARAM_SUBBAND_CHANS > 0 unless a shape was set;
+                                     with 17, inputs on which partial sums shared between trials
+                                     are estimated to be faster take the pattern-row kernel (same sums) */
 #define HP_PARAM_STAGE_TIMING 7   /* 1 = record CUDA events around every stage launch */
 #define HP_PARAM_TIMEOUT_S 8      /* limit of every bounded device wait, seconds (> 0) */
 #define HP_PARAM_RFI 9            /* 1 = RFI mitigation before dedispersion (default 0) */

@@ -89,6 +89,9 @@ struct DedispTiling {
     std::vector<StageDesc> stages;
     std::vector<ChanDesc> chans;
     std::vector<uint32_t> addr;    // per stage [pair][BD][2] byte offsets in the stage buffer
+                                   // (pattern rows: the stage tables of patterns.cuh)
+    bool pattern = false;          // tables of the pattern-row kernel (patterns.cu), with its
+    double cycles = 0;             // estimated SM cycles per time tile, summed over the DM tiles
     int64_t max_reach = 0;         // max over rows of goff + row bytes
 };
 
@@ -113,6 +116,7 @@ struct DedispJob {
     // left to the search.
     int32_t* lv;
     int64_t lv_pitch;
+    int64_t pattern;           // 1: tables of the pattern-row kernel
 };
 
 // Jobs of one dedispersion launch, passed by value as the kernel parameter.
@@ -158,6 +162,9 @@ cudaError_t launch_dedisp(int cfg, const DedispBatch& batch, int* status, uint64
 // and time tiles past a segment's needed length skip its stages.
 // Byte-row configs for which segmented_config() holds only.
 bool segmented_config(int cfg);
+// The jobs whose tables are the pattern-row kernel's (launch_dedisp sends them here).
+cudaError_t launch_dedisp_patterns(const DedispBatch& batch, int* status, uint64_t timeout_ns,
+                                   cudaStream_t s);
 cudaError_t launch_dedisp_segmented(int cfg, const DedispBatch& batch, int* status,
                                     uint64_t timeout_ns, cudaStream_t s);
 

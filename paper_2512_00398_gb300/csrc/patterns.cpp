@@ -1,0 +1,498 @@
+// patterns.cpp -- host tiling of the pattern-row dedispersion kernel
+// (patterns.cu): which consecutive channels are summed into shared rows, the
+// distinct delay patterns of every DM tile, and the stage tables.
+#include <algorithm>
+#include <atomic>
+#include <cstring>
+#include <thread>
+#include <vector>
+
+#include "patterns.cuh"
+#include "plan_internal.h"
+
+namespace hp {
+namespace {
+
+// One distinct pattern of a group: its channels' delays relative to the first
+// channel's, and the range of first-channel delays of the trials that use it.
+struct Pattern {
+    int32_t rel[kPatMaxGroup];
+    int32_t lo, hi;
+};
+
+struct Group {
+    int c = 0, n = 0;               // channels [c, c + n)
+    int32_t u0 = 0;                 // sample that chunk 0 starts at (first channel)
+    std::vector<Pattern> pats;
+    std::vector<int> of_trial;      // pattern of every trial
+    int32_t goff[kPatMaxGroup];     // staged window of every channel
+    uint32_t nwords[kPatMaxGroup];
+};
+
+int chunk_lo(const Pattern& q, int32_t u0) { return (q.lo - u0) / kPatChunk; }
+int chunk_hi(const Pattern& q, int32_t u0) {
+    return (q.hi - u0 + kPatL + kPatChunk - 1) / kPatChunk;
+}
+
+struct TileOut {
+    std::vector<StageDesc> stages;
+    std::vector<ChanDesc> chans;
+    std::vector<uint32_t> tab;
+    int64_t max_reach = 0;
+    double cost = 0;                // estimated SM cycles per time tile
+    bool ok = false;
+};
+
+struct TileBuilder {
+    const hp_plan* p;
+    int d0, nd;
+    bool strict;    // bound the tables of a group from above instead of estimating them
+
+    int32_t delay(int j, int c) const { return p->delays[(size_t)(d0 + j) * p->nchans + c]; }
+
+    // Estimated SM cycles of a group whose sets unpack `sets` chunks in all and put
+    // `rows` chunks into rows; fitted to 1620 cycles per group (15 and 51 chunks) at
+    // 4096 channels, 1700 (16, 56) at 2048 and 2320 (26, 88) at 1024, 24 trials each.
+    double group_cost(double sets, double rows) const {
+        return 150.0 + 21.0 * nd + 21.0 * sets + 13.0 * rows;
+    }
+
+    void make_group(int c, int n, Group* g) const {
+        g->c = c;
+        g->n = n;
+        g->pats.clear();
+        g->of_trial.assign(nd, 0);
+        int32_t lo = delay(0, c);
+        for (int j = 0; j < nd; ++j) {
+            Pattern q{};
+            for (int k = 0; k < n; ++k) q.rel[k] = delay(j, c + k) - delay(j, c);
+            q.lo = q.hi = delay(j, c);
+            lo = std::min(lo, q.lo);
+            size_t i = 0;
+            while (i < g->pats.size() && std::memcmp(g->pats[i].rel, q.rel, sizeof(q.rel))) ++i;
+            if (i == g->pats.size()) g->pats.push_back(q);
+            g->pats[i].lo = std::min(g->pats[i].lo, q.lo);
+            g->pats[i].hi = std::max(g->pats[i].hi, q.hi);
+            g->of_trial[j] = (int)i;
+        }
+        g->u0 = lo & ~3;
+        for (int k = 0; k < n; ++k) {
+            int32_t a = delay(0, c + k), b = a;
+            for (int j = 1; j < nd; ++j) {
+                a = std::min(a, delay(j, c + k));
+                b = std::max(b, delay(j, c + k));
+            }
+            g->goff[k] = a & ~15;
+            g->nwords[k] = (uint32_t)((b - g->goff[k] + kPatBT + 15) / 16 * 4);
+        }
+    }
+
+    // Slot of channel k of a group of n (PatItem).
+    static int slot(int n, int k) { return n > 2 ? k : 2 * k; }
+
+    // The set that starts at pattern i of the order: the patterns up to the returned
+    // index, whose shifts differ by no more than their slots allow (lo: the smallest
+    // positions in the channels' windows).
+    static size_t set_end(const Group& g, const std::vector<int>& ord, size_t i,
+                          int32_t (&lo)[kPatMaxGroup]) {
+        static const int limit[4] = {0, kPatShift1, kPatShift2, kPatShift2};
+        int32_t hi[kPatMaxGroup];
+        size_t e = i;
+        for (; e < ord.size(); ++e) {
+            int32_t l2[kPatMaxGroup], h2[kPatMaxGroup];
+            bool fits = true;
+            for (int k = 0; k < g.n; ++k) {
+                const int32_t at = g.u0 - g.goff[k] + g.pats[ord[e]].rel[k];
+                l2[k] = e == i ? at : std::min(lo[k], at);
+                h2[k] = e == i ? at : std::max(hi[k], at);
+                fits = fits && h2[k] - l2[k] <= limit[slot(g.n, k)];
+            }
+            if (!fits) break;
+            std::copy(l2, l2 + g.n, lo);
+            std::copy(h2, h2 + g.n, hi);
+        }
+        return e;
+    }
+
+    // One item of a set: its form cost (instructions, about) orders the items.
+    struct Item {
+        PatItem d;
+        std::vector<PatRow> rows;
+        int cost;
+    };
+
+    // The items of a group whose rows start at byte `row` of the row buffer and
+    // whose channels' windows start at chan_off in the raw buffer; org: per pattern
+    // the row buffer's byte offset of its word 0.
+    void make_items(const Group& g, const std::vector<int>& ord, const uint32_t* chan_off, uint32_t row,
+                    std::vector<Item>* items, std::vector<uint32_t>* org) const {
+        org->assign(g.pats.size(), 0);
+        for (size_t i = 0; i < ord.size();) {
+            int32_t lo[kPatMaxGroup];
+            const size_t e = set_end(g, ord, i, lo);
+            PatItem d{};
+            d.nchan = (uint8_t)g.n;
+            for (int k = 0; k < 4; ++k) d.off[k] = chan_off[0] + (uint32_t)(lo[0] & ~3);   // empty slots
+            for (int k = 0; k < g.n; ++k) {
+                d.off[slot(g.n, k)] = chan_off[k] + (uint32_t)(lo[k] & ~3);
+                d.sel[slot(g.n, k)] = (uint16_t)(0x3210u + 0x1111u * (uint32_t)(lo[k] & 3));
+            }
+            struct Row { int kind, lo, n; uint32_t row; };
+            std::vector<Row> rows;
+            int first = 1 << 30, last = 0;
+            for (; i < e; ++i) {
+                const Pattern& q = g.pats[ord[i]];
+                int shift[4] = {};
+                for (int k = 0; k < g.n; ++k)
+                    shift[slot(g.n, k)] = g.u0 - g.goff[k] + q.rel[k] - lo[k];
+                Row r;
+                r.kind = 9 * shift[1] + 3 * shift[2] + shift[3];
+                r.lo = chunk_lo(q, g.u0);
+                r.n = chunk_hi(q, g.u0) - r.lo;
+                r.row = row;
+                (*org)[ord[i]] = row - (uint32_t)r.lo * kPatChunk * 4;
+                row += (uint32_t)r.n * kPatChunk * 4;
+                first = std::min(first, r.lo);
+                last = std::max(last, r.lo + r.n);
+                rows.push_back(r);
+            }
+            // items of kPatItem chunks from the first chunk that any pattern covers
+            for (int c0 = first; c0 < last; c0 += kPatItem) {
+                Item it;
+                it.d = d;
+                for (int k = 0; k < 4; ++k) it.d.off[k] += (uint32_t)(c0 * kPatChunk);
+                it.cost = 200;
+                for (const Row& r : rows) {
+                    uint32_t put = 0;
+                    for (int q = 0; q < kPatItem; ++q)
+                        if (c0 + q >= r.lo && c0 + q < r.lo + r.n) put |= 1u << q;
+                    if (put == 0) continue;
+                    // (the item may start before the row; those chunks' stores are masked)
+                    it.rows.push_back(
+                        PatRow{r.row + (uint32_t)((c0 - r.lo + kPatItem - 1) * kPatChunk * 4),
+                               (uint16_t)put, (uint16_t)r.kind});
+                    it.cost += 32;
+                }
+                if (it.rows.empty()) continue;
+                it.d.nrows = (uint8_t)it.rows.size();
+                items->push_back(std::move(it));
+            }
+        }
+    }
+
+    static uint32_t items_bytes(const std::vector<Item>& items) {
+        uint32_t b = 0;
+        for (const Item& it : items) b += (uint32_t)(sizeof(PatItem) + it.rows.size() * sizeof(PatRow));
+        return b;
+    }
+
+    // The cheapest cut of the channels [begin, nch) into groups of 1 .. kPatMaxGroup.
+    bool cut(int begin, int nch, std::vector<uint8_t>* len, double* total) const {
+        std::vector<double> best(nch + 1, 0.0);
+        len->assign(nch, 0);
+        std::vector<int> cls(nd), next(nd);
+        std::vector<std::pair<int, int32_t>> keys;   // the patterns, by refinement
+        std::vector<int32_t> lo(nd), hi(nd);         // their ranges of first-channel delays
+        for (int c = nch - 1; c >= begin; --c) {
+            best[c] = 1e300;
+            std::fill(cls.begin(), cls.end(), 0);
+            int32_t u0 = delay(0, c);
+            for (int j = 1; j < nd; ++j) u0 = std::min(u0, delay(j, c));
+            u0 &= ~3;
+            uint32_t raw = 0;
+            int32_t range[kPatMaxGroup];       // of each channel's shift
+            for (int n = 1; n <= kPatMaxGroup && c + n <= nch; ++n) {
+                // refine the classes by the n-th channel
+                keys.clear();
+                int32_t a = delay(0, c + n - 1), b = a;
+                int32_t r_lo = a - delay(0, c), r_hi = r_lo;
+                for (int j = 0; j < nd; ++j) {
+                    const int32_t base = delay(j, c), v = delay(j, c + n - 1);
+                    a = std::min(a, v);
+                    b = std::max(b, v);
+                    r_lo = std::min(r_lo, v - base);
+                    r_hi = std::max(r_hi, v - base);
+                    const std::pair<int, int32_t> key(cls[j], v - base);
+                    size_t i = 0;
+                    while (i < keys.size() && keys[i] != key) ++i;
+                    if (i == keys.size()) {
+                        keys.push_back(key);
+                        lo[i] = hi[i] = base;
+                    }
+                    lo[i] = std::min(lo[i], base);
+                    hi[i] = std::max(hi[i], base);
+                    next[j] = (int)i;
+                }
+                cls = next;
+                raw += (uint32_t)((b - (a & ~15) + kPatBT + 15) / 16 * 16);
+                int chunks = 0, span = 0;
+                for (size_t i = 0; i < keys.size(); ++i) {
+                    Pattern q{};
+                    q.lo = lo[i];
+                    q.hi = hi[i];
+                    const int e = chunk_hi(q, u0);
+                    chunks += e - chunk_lo(q, u0);
+                    span = std::max(span, e);
+                }
+                // about as many sets as the widest range of shifts needs
+                range[n - 1] = r_hi - r_lo;
+                double sets = 1.0;
+                for (int k = 1; k < n; ++k)
+                    sets = std::max(sets, (range[k] + 1.0) / (slot(n, k) == 1 ? kPatShift1 + 1 : kPatShift2 + 1));
+                // (strict: every pattern in a set of its own)
+                const double items = strict ? chunks / kPatItem + 2 * keys.size()
+                                            : 1.3 * sets * (span / kPatItem + 1);
+                const double tab = sizeof(PatHeader) + items * sizeof(PatItem) +
+                                   (chunks / kPatItem + 2 * keys.size()) * sizeof(PatRow);
+                if ((size_t)chunks * kPatChunk * 4 > (size_t)kPatRowBytes ||
+                    raw > (uint32_t)(kPatRawBytes - kPatTabBytes) || tab > kPatTabBytes - 16)
+                    break;   // more channels only add to each
+                const double cost = group_cost(sets * (span + 1), chunks) + best[c + n];
+                if (cost < best[c]) {
+                    best[c] = cost;
+                    (*len)[c] = (uint8_t)n;
+                }
+            }
+            if ((*len)[c] == 0) return false;
+        }
+        *total = best[begin];
+        return true;
+    }
+
+    void build(TileOut* out) const {
+        std::vector<uint8_t> len;
+        const int nch = p->nchans;
+        if (!cut(0, nch, &len, &out->cost)) return;
+        // the stage being packed
+        std::vector<Item> items;
+        std::vector<uint32_t> trials;
+        StageDesc sd{};
+        uint32_t rows = 0, raw = kPatTabBytes, tab = sizeof(PatHeader);
+        int groups = 0, held = 0;
+        std::vector<int64_t> load(kPatFormWarps, 0);   // cost given to every forming warp so far
+        size_t last_trials = 0;                        // trial table of the last stage emitted
+        auto flush_last = [&]() {
+            PatTrials h;
+            std::memcpy(&h, &out->tab[last_trials], sizeof(h));
+            h.flush = 1;
+            std::memcpy(&out->tab[last_trials], &h, sizeof(h));
+        };
+        auto emit = [&]() {
+            if (held + (int)sd.nchan > kStageMaxChans) {   // the stage before flushes
+                flush_last();
+                held = 0;
+            }
+            held += (int)sd.nchan;
+            // the costliest items first, each to the warp with the least work so far
+            std::stable_sort(items.begin(), items.end(),
+                             [](const Item& x, const Item& y) { return x.cost > y.cost; });
+            std::vector<std::vector<int>> of(kPatFormWarps);
+            std::vector<int64_t> here(kPatFormWarps, 0);
+            for (size_t i = 0; i < items.size(); ++i) {
+                int w = 0;
+                for (int v = 1; v < kPatFormWarps; ++v)
+                    if (std::make_pair(here[v], load[v]) < std::make_pair(here[w], load[w])) w = v;
+                of[w].push_back((int)i);
+                here[w] += items[i].cost;
+                load[w] += items[i].cost;
+            }
+            tab = (tab + 15) & ~15u;       // copied in 16-byte pieces
+            sd.addr_begin = (uint32_t)out->tab.size();
+            sd.addr_bytes = tab;
+            sd.addr_off = (uint32_t)(sizeof(PatTrials) + trials.size() * 4);
+            sd.tx_bytes += tab + sd.addr_off;
+            out->tab.resize(out->tab.size() + (sd.addr_bytes + sd.addr_off) / 4);
+            uint8_t* base = reinterpret_cast<uint8_t*>(&out->tab[sd.addr_begin]);
+            PatHeader h{};
+            uint32_t n = 0, b_off = (uint32_t)(sizeof(h) + items.size() * sizeof(PatItem));
+            for (int w = 0; w < kPatFormWarps; ++w) {
+                h.begin[w] = (uint8_t)n;
+                for (int i : of[w]) {
+                    Item& it = items[i];
+                    it.d.row_off = (uint16_t)b_off;
+                    std::memcpy(base + sizeof(h) + n * sizeof(PatItem), &it.d, sizeof(PatItem));
+                    std::memcpy(base + b_off, it.rows.data(), it.rows.size() * sizeof(PatRow));
+                    b_off += (uint32_t)(it.rows.size() * sizeof(PatRow));
+                    ++n;
+                }
+            }
+            h.begin[kPatFormWarps] = (uint8_t)n;
+            std::memcpy(base, &h, sizeof(h));
+            PatTrials th{};
+            th.ngroups = (uint32_t)groups;
+            std::memcpy(base + tab, &th, sizeof(th));
+            std::memcpy(base + tab + sizeof(th), trials.data(), trials.size() * 4);
+            last_trials = sd.addr_begin + tab / 4;
+            out->stages.push_back(sd);
+            items.clear();
+            trials.clear();
+            rows = 0;
+            raw = kPatTabBytes;
+            tab = sizeof(PatHeader);
+            groups = 0;
+        };
+        Group g;
+        std::vector<int> ord;
+        std::vector<Item> more;
+        std::vector<uint32_t> org;
+        for (int c = 0; c < nch; c += len[c]) {
+            make_group(c, len[c], &g);
+            ord.resize(g.pats.size());
+            for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int)i;
+            std::sort(ord.begin(), ord.end(), [&](int x, int y) {
+                return std::lexicographical_compare(g.pats[x].rel, g.pats[x].rel + g.n, g.pats[y].rel,
+                                                    g.pats[y].rel + g.n);
+            });
+            uint32_t grows = 0, graw = 0;
+            for (const Pattern& q : g.pats)
+                grows += (uint32_t)(chunk_hi(q, g.u0) - chunk_lo(q, g.u0)) * kPatChunk * 4;
+            for (int k = 0; k < g.n; ++k) graw += 4 * g.nwords[k];
+            uint32_t chan_off[kPatMaxGroup] = {};
+            auto lay = [&]() {
+                uint32_t at = raw;
+                for (int k = 0; k < g.n; ++k) {
+                    chan_off[k] = at;
+                    at += 4 * g.nwords[k];
+                }
+                more.clear();
+                make_items(g, ord, chan_off, rows, &more, &org);
+            };
+            lay();
+            if (groups > 0 && (groups == kPatStageGroups || rows + grows > (uint32_t)kPatRowBytes ||
+                               raw + graw > (uint32_t)kPatRawBytes ||
+                               tab + items_bytes(more) + 15 > (uint32_t)kPatTabBytes ||
+                               items.size() + more.size() > 255)) {
+                emit();
+                lay();
+            }
+            if (items_bytes(more) + tab + 15 > (uint32_t)kPatTabBytes || more.size() > 255) return;
+            if (groups == 0) {
+                sd = StageDesc{};
+                sd.chan_begin = (uint32_t)out->chans.size();
+            }
+            for (int k = 0; k < g.n; ++k) {
+                ChanDesc cd;
+                cd.c = (uint32_t)(g.c + k);
+                cd.goff = g.goff[k];
+                cd.offB = chan_off[k];
+                cd.nwords = g.nwords[k];
+                out->chans.push_back(cd);
+                sd.tx_bytes += 4 * g.nwords[k];
+                out->max_reach = std::max<int64_t>(out->max_reach, (int64_t)g.goff[k] + 4 * g.nwords[k]);
+            }
+            sd.nchan += (uint32_t)g.n;
+            trials.resize(trials.size() + kPatSumWarps * kPatPlaces);
+            uint32_t* t = &trials[trials.size() - kPatSumWarps * kPatPlaces];
+            for (int j = 0; j < kPatBD; ++j) {
+                const int jj = j < nd ? j : 0;
+                t[j / kPatRD * kPatPlaces + j % kPatRD] =
+                    org[g.of_trial[jj]] + 4u * (uint32_t)(delay(jj, g.c) - g.u0);
+            }
+            tab += items_bytes(more);
+            for (Item& it : more) items.push_back(std::move(it));
+            rows += grows;
+            raw += graw;
+            ++groups;
+        }
+        emit();
+        flush_last();
+        out->ok = true;
+    }
+};
+
+}  // namespace
+
+bool parallel_for(int n, int threads, const std::function<void(int)>& f) {
+    std::atomic<int> next{0};
+    std::atomic<bool> failed{false};
+    auto work = [&]() {
+        try {
+            for (int i; !failed && (i = next++) < n;) f(i);
+        } catch (...) {
+            failed = true;
+        }
+    };
+    const int want = std::min({n, threads, (int)std::max(1u, std::thread::hardware_concurrency())});
+    std::vector<std::thread> pool;
+    try {
+        for (int i = 1; i < want; ++i) pool.emplace_back(work);
+    } catch (...) {   // fewer threads than wanted
+    }
+    work();
+    for (std::thread& t : pool) t.join();
+    return !failed;
+}
+
+// 83 sums per SM and cycle (1.61 M cycles per block of 15 trials x 2176 samples on
+// the 4096-channel file; 82 at 1024 channels).
+double byte_row_cycles(double sums) { return sums / 83.0; }
+
+// First trial of DM tile i.
+static int pattern_tile(int ndm, int ntiles, int i) { return (int)((int64_t)ndm * i / ntiles); }
+
+double estimate_patterns(const hp_plan* p) {
+    const int ndm = p->ndm(), ntiles = (ndm + kPatBD - 1) / kPatBD;
+    const int nd = std::min(ntiles, 3), nc = std::min(p->nchans / 8 + 1, 8);
+    double sum = 0;
+    std::vector<uint8_t> len;
+    try {
+        for (int i = 0; i < nd; ++i) {
+            const int t = (int)((2 * i + 1) * (int64_t)ntiles / (2 * nd));
+            const int d0 = pattern_tile(ndm, ntiles, t);
+            const TileBuilder b{p, d0, pattern_tile(ndm, ntiles, t + 1) - d0, false};
+            for (int j = 0; j < nc; ++j) {
+                const int c = (int)((2 * j + 1) * (int64_t)p->nchans / (2 * nc)) / 8 * 8;
+                const int e = std::min(c + 8, p->nchans);
+                double cycles = 0;
+                if (!b.cut(c, e, &len, &cycles)) return -1;
+                sum += cycles / (e - c);
+            }
+        }
+    } catch (...) {
+        return -1;
+    }
+    return sum / (nd * nc) * p->nchans * ntiles;
+}
+
+bool build_patterns(const hp_plan* p, DedispTiling* T) {
+    const int ndm = p->ndm(), ntiles = (ndm + kPatBD - 1) / kPatBD;
+    std::atomic<bool> failed{false};
+    try {
+        std::vector<DedispTiling> parts(ntiles);
+        std::vector<double> cycles(ntiles, 0.0);
+        // one thread per 1024 channels of a tile (about 1 ms)
+        const int threads = (int)std::min<int64_t>((int64_t)ntiles * p->nchans / 1024, 16);
+        const bool done = parallel_for(ntiles, threads, [&](int i) {
+            if (failed) return;
+            const int d0 = pattern_tile(ndm, ntiles, i), d1 = pattern_tile(ndm, ntiles, i + 1);
+            TileOut out;
+            for (int strict = 0; strict < 2 && !out.ok; ++strict) {
+                out = TileOut();
+                TileBuilder{p, d0, d1 - d0, strict != 0}.build(&out);
+            }
+            if (!out.ok) {
+                failed = true;
+                return;
+            }
+            DedispTiling& q = parts[i];
+            q.tiles.push_back(TileDesc{d0, d1 - d0, 0, (int32_t)out.stages.size()});
+            q.stages.swap(out.stages);
+            q.chans.swap(out.chans);
+            q.addr.swap(out.tab);
+            q.max_reach = out.max_reach;
+            cycles[i] = out.cost;
+        });
+        if (!done || failed) return false;
+        append_tiling(parts, T);
+        for (double c : cycles) T->cycles += c;
+    } catch (...) {
+        *T = DedispTiling();
+        return false;
+    }
+    T->BD = kPatBD;
+    T->BT = kPatBT;
+    T->pattern = true;
+    return true;
+}
+
+}  // namespace hp

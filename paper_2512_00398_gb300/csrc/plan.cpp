@@ -11,6 +11,7 @@
 #include <new>
 #include <vector>
 
+#include "patterns.cuh"
 #include "plan_internal.h"
 
 using namespace hp;
@@ -237,6 +238,34 @@ int append_tile(const Delay& delay, int nd, int nch, const std::vector<int>& seg
     return HP_OK;
 }
 
+void append_tiling(std::vector<DedispTiling>& parts, DedispTiling* T) {
+    size_t st = 0, ch = 0, ad = 0;
+    for (const DedispTiling& q : parts) {
+        st += q.stages.size();
+        ch += q.chans.size();
+        ad += q.addr.size();
+    }
+    T->stages.reserve(st);
+    T->chans.reserve(ch);
+    T->addr.reserve(ad);
+    for (DedispTiling& q : parts) {
+        for (TileDesc td : q.tiles) {
+            td.stage_begin += (int32_t)T->stages.size();
+            T->tiles.push_back(td);
+        }
+        const uint32_t c0 = (uint32_t)T->chans.size(), a0 = (uint32_t)T->addr.size();
+        for (StageDesc sd : q.stages) {
+            sd.chan_begin += c0;
+            sd.addr_begin += a0;
+            T->stages.push_back(sd);
+        }
+        T->chans.insert(T->chans.end(), q.chans.begin(), q.chans.end());
+        T->addr.insert(T->addr.end(), q.addr.begin(), q.addr.end());
+        T->max_reach = std::max(T->max_reach, q.max_reach);
+        q = DedispTiling();
+    }
+}
+
 // The nominal trial of the group of trial d (sub-band variant): the lower
 // middle trial of the group.
 int sb_nominal(const hp_plan* p, int d) {
@@ -290,23 +319,32 @@ int build_tiling(hp_plan* p, int cfg, DedispTiling* T) {
         T->cfg = cfg;
         return HP_OK;
     }
-    int d0 = 0;
-    while (d0 < ndm) {
-        // grow the tile while every channel row alone still fits a stage
-        int nd = 1;
-        while (nd < BD && d0 + nd < ndm) {
-            bool ok = true;
-            for (int c = nch - 1; c >= 0 && ok; --c)
-                ok = row_geom(p, d0, nd + 1, c, BT).smem + stage_header(1, BD) <= budget;
-            if (!ok) break;
-            ++nd;
-        }
-        const int32_t* base = &p->delays[(size_t)d0 * nch];
-        auto delay = [&](int j, int c) { return base[(size_t)j * nch + c]; };
-        const int rc = append_tile(delay, nd, nch, {0}, {d0}, {0u}, d0, C, T);
-        if (rc) return rc;
-        d0 += nd;
+    // tile boundaries: BD trials, fewer where a channel row of that many would not
+    // fit a stage alone (a row only grows with the trials it serves)
+    auto fits = [&](int d, int nd) {
+        for (int c = nch - 1; c >= 0; --c)
+            if (row_geom(p, d, nd, c, BT).smem + stage_header(1, BD) > budget) return false;
+        return true;
+    };
+    std::vector<int> first{0};
+    while (first.back() < ndm) {
+        const int d0 = first.back();
+        int nd = std::min(BD, ndm - d0);
+        while (nd > 1 && !fits(d0, nd)) --nd;
+        first.push_back(d0 + nd);
     }
+    const int ntiles = (int)first.size() - 1;
+    std::vector<DedispTiling> part(ntiles);   // (threads: about 0.5 ms of work each)
+    std::vector<int> rcs(ntiles, HP_OK);
+    const bool done = parallel_for(ntiles, (int)std::min<int64_t>((int64_t)ntiles * nch / 8192, 16), [&](int i) {
+        const int32_t* base = &p->delays[(size_t)first[i] * nch];
+        auto delay = [&](int j, int c) { return base[(size_t)j * nch + c]; };
+        rcs[i] = append_tile(delay, first[i + 1] - first[i], nch, {0}, {first[i]}, {0u}, first[i], C, &part[i]);
+    });
+    if (!done) return HP_ERR_OOM;
+    for (int rc : rcs)
+        if (rc) return rc;
+    append_tiling(part, T);
     T->cfg = cfg;
     return HP_OK;
 }
@@ -546,6 +584,8 @@ int ensure_device_tables(hp_plan* p) {
         int rc = build_tiling(p, p->dedisp_cfg, &p->tiling);
         if (rc) return rc;
     }
+    if (cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return HP_ERR_CUDA;
     const DedispTiling& T = p->tiling;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -581,21 +621,21 @@ int ensure_device_tables(hp_plan* p) {
     void* mem = nullptr;
     int rc = plan_alloc(p, total, &mem);
     if (rc) return rc;
-    std::vector<uint8_t> host(total, 0);
-    std::memcpy(host.data() + o_status, &prev_status, sizeof(int));
-    std::memcpy(host.data() + o_tiles, T.tiles.data(), T.tiles.size() * sizeof(TileDesc));
-    std::memcpy(host.data() + o_stages, T.stages.data(), T.stages.size() * sizeof(StageDesc));
-    std::memcpy(host.data() + o_chans, T.chans.data(), T.chans.size() * sizeof(ChanDesc));
-    std::memcpy(host.data() + o_addr, T.addr.data(), T.addr.size() * sizeof(uint32_t));
-    std::memcpy(host.data() + o_widths, p->widths.data(), p->widths.size() * sizeof(int32_t));
-    if (!sbtop.empty())
-        std::memcpy(host.data() + o_sbtop, sbtop.data(), sbtop.size() * sizeof(int32_t));
-    rc = check_cuda(cudaMemcpy(mem, host.data(), total, cudaMemcpyHostToDevice));
+    uint8_t* b = (uint8_t*)mem;
+    auto put = [&](size_t at, const void* src, size_t bytes) {
+        if (!rc && bytes) rc = check_cuda(cudaMemcpy(b + at, src, bytes, cudaMemcpyHostToDevice));
+    };
+    put(o_status, &prev_status, sizeof(int));
+    put(o_tiles, T.tiles.data(), T.tiles.size() * sizeof(TileDesc));
+    put(o_stages, T.stages.data(), T.stages.size() * sizeof(StageDesc));
+    put(o_chans, T.chans.data(), T.chans.size() * sizeof(ChanDesc));
+    put(o_addr, T.addr.data(), T.addr.size() * sizeof(uint32_t));
+    put(o_widths, p->widths.data(), p->widths.size() * sizeof(int32_t));
+    put(o_sbtop, sbtop.data(), sbtop.size() * sizeof(int32_t));
     if (rc) {
         plan_free(p, mem, total);
         return rc;
     }
-    uint8_t* b = (uint8_t*)mem;
     p->tables = mem;
     p->tables_bytes = total;
     p->tables_cfg = p->dedisp_cfg;
@@ -639,23 +679,102 @@ bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch) {
     return last_t0 + p->tiling.max_reach <= xt_pitch;
 }
 
+// Is a launch of njobs inputs of nout samples faster with pattern rows that take
+// `cycles` per time tile?  Both kernels keep one block per SM, so the one whose last
+// wave ends first, by the estimated cycles of its blocks: the pattern rows' larger
+// tiles (24 trials x 2048 samples against 15 x 2176) lose on short inputs, where a
+// wave is nearly empty, although they take fewer cycles per sum.  (The 1.03 leaves
+// near ties, within the estimates' error, to the byte rows.)
+bool patterns_pay(const hp_plan* p, double cycles, int64_t nout, int njobs) {
+    // the default tile shape of direct dedispersion, without fused remedian levels
+    if (p->dedisp_cfg != kDefaultDedispConfig || p->sb_chans > 0 || p->fuse_levels) return false;
+    if (cycles <= 0 || nout <= 0) return false;
+    const DedispTiling& T = p->tiling;
+    const int64_t nt = (int64_t)T.tiles.size(), nq = ceil_div(p->ndm(), kPatBD);
+    const double q = (double)ceil_div(ceil_div(nout, kPatBT) * nq * njobs, p->sm_count) * cycles / (double)nq;
+    const double t = (double)ceil_div(ceil_div(nout, T.BT) * nt * njobs, p->sm_count) *
+                     byte_row_cycles((double)T.BD * p->nchans * T.BT);
+    return q * 1.03 < t;
+}
+
+bool use_patterns(const hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs) {
+    const DedispTiling& Q = p->ptiling;
+    return p->ptables && (ceil_div(nout, Q.BT) - 1) * Q.BT + Q.max_reach <= xt_pitch &&
+           patterns_pay(p, Q.cycles, nout, njobs);
+}
+
+int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s) {
+    if (p->ptables || p->pat_estimate < 0 || p->dedisp_cfg != kDefaultDedispConfig ||
+        p->sb_chans > 0 || p->fuse_levels)
+        return HP_OK;
+    if (p->pat_estimate == 0) p->pat_estimate = estimate_patterns(p);
+    if (!patterns_pay(p, p->pat_estimate, nout, njobs)) return HP_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return HP_OK;
+    DedispTiling& Q = p->ptiling;
+    if (!Q.pattern && !build_patterns(p, &Q)) {
+        p->pat_estimate = -1;
+        return HP_OK;
+    }
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        size_t at = off;
+        off = align_up(off + bytes, 256);
+        return at;
+    };
+    const size_t o_tiles = take(Q.tiles.size() * sizeof(TileDesc));
+    const size_t o_stages = take(Q.stages.size() * sizeof(StageDesc));
+    const size_t o_chans = take(Q.chans.size() * sizeof(ChanDesc));
+    const size_t o_addr = take(Q.addr.size() * sizeof(uint32_t));
+    void* mem = nullptr;
+    int rc = plan_alloc(p, off, &mem);
+    if (rc) return HP_OK;   // no room: the byte rows run
+    uint8_t* b = (uint8_t*)mem;
+    auto put = [&](size_t at, const void* src, size_t bytes) {
+        if (!rc) rc = check_cuda(cudaMemcpy(b + at, src, bytes, cudaMemcpyHostToDevice));
+    };
+    put(o_tiles, Q.tiles.data(), Q.tiles.size() * sizeof(TileDesc));
+    put(o_stages, Q.stages.data(), Q.stages.size() * sizeof(StageDesc));
+    put(o_chans, Q.chans.data(), Q.chans.size() * sizeof(ChanDesc));
+    put(o_addr, Q.addr.data(), Q.addr.size() * sizeof(uint32_t));
+    if (rc) {
+        plan_free(p, mem, off);
+        return rc;
+    }
+    // (the host needs only the tile list, the extents and the estimate from now on)
+    std::vector<StageDesc>().swap(Q.stages);
+    std::vector<ChanDesc>().swap(Q.chans);
+    std::vector<uint32_t>().swap(Q.addr);
+    p->ptables = mem;
+    p->ptables_bytes = off;
+    p->d_ptiles = (const TileDesc*)(b + o_tiles);
+    p->d_pstages = (const StageDesc*)(b + o_stages);
+    p->d_pchans = (const ChanDesc*)(b + o_chans);
+    p->d_paddr = (const uint32_t*)(b + o_addr);
+    return HP_OK;
+}
+
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
-                   int64_t out_pitch, int64_t nout) {
+                   int64_t out_pitch, int64_t nout, int njobs) {
     DedispJob J;
+    const bool pat = use_patterns(p, nout, xt_pitch, njobs);
+    const DedispTiling& T = pat ? p->ptiling : p->tiling;
     J.xt = xt;
     J.xt_pitch = xt_pitch;
     J.out = out;
     J.out_pitch = out_pitch;
     J.nout = nout;
-    J.ntt = (int32_t)ceil_div(nout, p->tiling.BT);
-    J.ndt = (int32_t)p->tiling.tiles.size();
-    if (!reach_ok(p, nout, xt_pitch)) J.ntt = J.ndt = 0;   // callers report the error
-    J.tiles = p->d_tiles;
-    J.stages = p->d_stages;
-    J.chans = p->d_chans;
-    J.addr = p->d_addr;
+    J.ntt = (int32_t)ceil_div(nout, T.BT);
+    J.ndt = (int32_t)T.tiles.size();
+    if (!pat && !reach_ok(p, nout, xt_pitch)) J.ntt = J.ndt = 0;   // callers report the error
+    J.tiles = pat ? p->d_ptiles : p->d_tiles;
+    J.stages = pat ? p->d_pstages : p->d_stages;
+    J.chans = pat ? p->d_pchans : p->d_chans;
+    J.addr = pat ? p->d_paddr : p->d_addr;
     J.lv = nullptr;
     J.lv_pitch = 0;
+    J.pattern = pat ? 1 : 0;
     return J;
 }
 
@@ -752,6 +871,8 @@ int run_dedisp(hp_plan* p, const uint8_t* fb, int64_t nsamps, const Layout& L, u
         if (rc) return rc;
     }
     if (p->sb_chans > 0) return run_subband(p, L, ws, out, out_pitch, s);
+    rc = prepare_patterns(p, nout, xt_pitch, 1, s);
+    if (rc) return rc;
     DedispBatch B;   // copied into the kernel parameters at launch
     std::memset(&B, 0, sizeof(B));
     B.njobs = 1;
@@ -998,7 +1119,7 @@ void batch_drop_graph(hp_batch* b) {
     b->seen = 0;
 }
 
-int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
+int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps, cudaStream_t s,
                   std::vector<Layout>* layouts, std::vector<uint8_t*>* wss) {
     const int n = (int)b->plans.size();
     layouts->resize(n);
@@ -1011,6 +1132,8 @@ int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
         rc = ensure_device_tables(p);
         if (rc) return rc;
         (*layouts)[i] = make_layout(p, nsamps[i], true);
+        rc = prepare_patterns(p, (*layouts)[i].nout, (*layouts)[i].xt_pitch, 1, s);
+        if (rc) return rc;
         rc = ensure_workspace(p, (*layouts)[i].total, &(*wss)[i]);
         if (rc) return rc;
     }
@@ -1119,6 +1242,7 @@ std::vector<uintptr_t> batch_key(const hp_batch* b, const uint8_t* const* fbs,
         k.push_back((uintptr_t)outs[i].count);
         k.push_back((uintptr_t)wss[i]);
         k.push_back((uintptr_t)p->tables);
+        k.push_back((uintptr_t)p->ptables);
         k.push_back((uintptr_t)p->baseline_mode);
         k.push_back((uintptr_t)(p->baseline_s * 1e9));
         k.push_back((uintptr_t)p->dm_tol);
@@ -1133,6 +1257,7 @@ std::vector<uintptr_t> batch_key(const hp_batch* b, const uint8_t* const* fbs,
         k.push_back((uintptr_t)p->sb_chans);
         k.push_back((uintptr_t)p->decimate);
         k.push_back((uintptr_t)p->sb_group);
+        k.push_back((uintptr_t)p->fuse_levels);
     }
     return k;
 }
@@ -1201,8 +1326,9 @@ int hp_plan_destroy(hp_plan* p) {
     if (!p) return HP_OK;
     bool any_ev = false;
     for (int st = 0; st < HP_NUM_STAGES; ++st) any_ev = any_ev || !p->ev[st].empty();
-    if (p->tables || p->ws_own || any_ev) cudaDeviceSynchronize();
+    if (p->tables || p->ptables || p->ws_own || any_ev) cudaDeviceSynchronize();
     plan_free(p, p->tables, p->tables_bytes);
+    plan_free(p, p->ptables, p->ptables_bytes);
     plan_free(p, p->ws_own, p->ws_own_bytes);
     for (int st = 0; st < HP_NUM_STAGES; ++st)
         for (cudaEvent_t e : p->ev[st]) cudaEventDestroy(e);
@@ -1341,13 +1467,17 @@ int hp_plan_workspace_bytes(const hp_plan* p, int64_t nsamps, size_t* bytes) {
 
 int hp_plan_set_allocator(hp_plan* p, hp_alloc_fn alloc, hp_free_fn free_fn, void* ctx) {
     if (!p || (alloc == nullptr) != (free_fn == nullptr)) return HP_ERR_INVALID_ARG;
-    if (p->tables || p->ws_own) {
+    if (p->tables || p->ptables || p->ws_own) {
         // return what the previous allocator gave (the tables keep the status word)
         int st = 0;
         if (p->status) cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost);
         cudaDeviceSynchronize();
         plan_free(p, p->tables, p->tables_bytes);
+        plan_free(p, p->ptables, p->ptables_bytes);
         plan_free(p, p->ws_own, p->ws_own_bytes);
+        p->ptables = nullptr;
+        p->ptables_bytes = 0;
+        p->ptiling = DedispTiling();   // built again on the next use
         p->tables = nullptr;
         p->tables_bytes = 0;
         p->tables_cfg = -1;
@@ -1616,7 +1746,7 @@ int hp_batch_search(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamp
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<Layout> Ls;
     std::vector<uint8_t*> wss;
-    int rc = batch_prepare(b, fbs, nsamps, &Ls, &wss);
+    int rc = batch_prepare(b, fbs, nsamps, s, &Ls, &wss);
     if (rc) return rc;
     const std::vector<uintptr_t> key = batch_key(b, fbs, nsamps, s, outs, wss);
     if (key != b->key) {
@@ -1668,7 +1798,7 @@ int hp_batch_autotune(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsa
         b->cfg = c;
         std::vector<Layout> Ls;
         std::vector<uint8_t*> wss;
-        rc = batch_prepare(b, fbs, nsamps, &Ls, &wss);
+        rc = batch_prepare(b, fbs, nsamps, s, &Ls, &wss);
         if (rc == HP_ERR_INVALID_ARG) { rc = HP_OK; continue; }
         if (rc) break;
         TransposeBatch tb;

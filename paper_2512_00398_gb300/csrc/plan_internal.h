@@ -5,6 +5,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <functional>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -81,6 +82,14 @@ struct hp_plan {
     const int32_t* d_sbtop = nullptr;
 
     hp::DedispTiling tiling;           // for dedisp_cfg
+    // Pattern-row tables, beside those of the default tile shape: built by the first
+    // input that the pattern-row kernel is estimated to be faster on.
+    hp::DedispTiling ptiling;
+    double pat_estimate = 0;           // SM cycles per time tile, all DM tiles, from a few of them
+                                       // (0: not estimated yet, < 0: no tables can be laid out)
+    void* ptables = nullptr;
+    size_t ptables_bytes = 0;
+    int sm_count = 148;
 
     // device state
     int device = -1;
@@ -93,6 +102,10 @@ struct hp_plan {
     const hp::StageDesc* d_stages = nullptr;
     const hp::ChanDesc* d_chans = nullptr;
     const uint32_t* d_addr = nullptr;
+    const hp::TileDesc* d_ptiles = nullptr;      // of ptiling
+    const hp::StageDesc* d_pstages = nullptr;
+    const hp::ChanDesc* d_pchans = nullptr;
+    const uint32_t* d_paddr = nullptr;
     int32_t* d_widths = nullptr;
 
     // device allocator for the plan's tables and workspace (default cudaMalloc)
@@ -131,12 +144,30 @@ int plan_alloc(hp_plan* p, size_t bytes, void** out);
 void plan_free(hp_plan* p, void* ptr, size_t bytes);
 int ensure_device_tables(hp_plan* p);
 int ensure_workspace(hp_plan* p, size_t need, uint8_t** base);
+// Tables of the pattern-row kernel for the plan's direct delays; false (T left
+// empty) where they cannot be laid out.
+bool build_patterns(const hp_plan* p, DedispTiling* T);
+// Its SM cycles per time tile, summed over the DM tiles, from a sample of the tiles
+// and channels; < 0 where a channel cannot be laid out.
+double estimate_patterns(const hp_plan* p);
+// Build the pattern-row tables if a launch of njobs inputs of nout samples is
+// estimated to be faster with them and s is not being captured (nothing can be
+// allocated then; the byte rows run).
+int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s);
+// Append the tiles of every part, whose indices count from its own tables (left empty).
+void append_tiling(std::vector<DedispTiling>& parts, DedispTiling* T);
+// Estimated SM cycles of the byte-row kernel for `sums` (trial, channel, sample) sums.
+double byte_row_cycles(double sums);
+// f(i) for i in [0, n) on up to `threads` host threads; false if one threw.
+bool parallel_for(int n, int threads, const std::function<void(int)>& f);
 Layout make_layout(const hp_plan* p, int64_t nsamps, bool with_dedisp);
 int64_t xt_pitch_for(int64_t nsamps);
 int validate_search_input(const hp_plan* p, const void* ptr, int64_t nsamps);
 bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch);
+// One job of a launch of about `njobs` such jobs (the choice between the byte-row
+// and the pattern-row kernel depends on how many blocks the launch has).
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
-                   int64_t out_pitch, int64_t nout);
+                   int64_t out_pitch, int64_t nout, int njobs = 1);
 // Stages 1 and 2 of the sub-band variant on the transposed input at ws + L.xt.
 int run_subband(hp_plan* p, const Layout& L, uint8_t* ws, int32_t* out, int64_t out_pitch,
                 cudaStream_t s);

@@ -295,7 +295,8 @@ int enqueue_step(hp_stream* s, Step* st) {
         tb.prefix[j + 1] = tb.prefix[j] + J.ttiles * J.ctiles;
         if (p->sb_chans <= 0) {   // the sub-band variant runs its own two stages per gulp
             if (!reach_ok(p, L.nout, L.xt_pitch)) return HP_ERR_INVALID_ARG;
-            db.jobs[j] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout);
+            db.jobs[j] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout,
+                                  (int)st->items.size());
             fuse_levels(db.jobs[j], L, ws);
             db.prefix[j + 1] = db.prefix[j] + (int64_t)db.jobs[j].ntt * db.jobs[j].ndt;
         }
@@ -484,8 +485,11 @@ int hp_stream_open(hp_stream** out, const hp_plan* tmpl, const hp_stream_config*
     int mb = cfg->max_batch ? cfg->max_batch : std::min(cfg->nbeams, HP_BATCH_MAX_FILES);
     mb = std::min(mb, cfg->nbeams);
     int slots = cfg->nbeams;
+    // (a gulp's window and the look-ahead of the widest boxcar)
+    rc = prepare_patterns(p, s->G + p->wmax - 1, L.xt_pitch, mb, nullptr);
+    if (rc) { release(s); return rc; }
     if (cfg->hbm_budget > 0) {
-        const int64_t avail = cfg->hbm_budget - (int64_t)p->tables_bytes;
+        const int64_t avail = cfg->hbm_budget - (int64_t)(p->tables_bytes + p->ptables_bytes);
         const int64_t step1 = (int64_t)(s->ws_bytes + s->cand_dev_bytes);
         while (mb >= 1 && mb * step1 + (int64_t)s->beam_bytes > avail) --mb;
         if (mb < 1) { release(s); return HP_ERR_OOM; }
