@@ -135,6 +135,32 @@ __device__ __forceinline__ void named_barrier_arrive(int id, int nthreads) {
     asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
+// Programmatic dependent launch: a kernel launched by launch_pdl starts while the
+// kernel before it in the stream still runs and calls pdl_wait before it touches
+// anything that one may write (pdl_wait returns once it is complete and its writes
+// are visible), then lets the next one start.  Short kernels follow each other
+// without the launch gap.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                       cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Floor division for a positive divisor.
 __device__ __forceinline__ long long floor_div_pos(long long a, long long b) {
     long long q = a / b;

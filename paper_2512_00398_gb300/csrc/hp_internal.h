@@ -332,7 +332,7 @@ struct MergeArgs {
     int32_t* dm_hi;
     unsigned long long* t_lo;
     unsigned long long* t_hi;
-    int32_t* scan;             // [cap]
+    int32_t* scan;             // [cap]: work counters of the general path
     int32_t* block_sums;       // [cap / 1024 + 1]
     int64_t* n_clamped;        // one int64
     int64_t* trial_start;      // [ndm + 1]: first sorted entry of each trial, or null
@@ -343,7 +343,5 @@ struct MergeArgs {
     int* status;
 };
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t s, int64_t* nlaunch);
-
-int merge_sort_passes(int64_t cap);
 
 }  // namespace hp

@@ -113,7 +113,7 @@ extern "C" int hp_merge_static(const hp_raw_cand* raw_dev, const int64_t* nraw_d
     // Every scratch word the merge kernels read is written earlier in the same
     // call (keys, union-find state, cluster statistics, scan sums), so nothing
     // left by a previous call needs clearing.
-    MergeArgs m;
+    MergeArgs m{};
     m.raw = raw_dev;
     m.nraw = nraw_dev;
     m.cap = raw_capacity;
