@@ -985,13 +985,22 @@ __global__ void __launch_bounds__(kDetectThreads) detect_kernel(const __grid_con
 //   max_i S_W(k + i) <= P[k + W] - P[k] + M+(k + W) - M-(k),
 // so one add and a sign test clear the whole group and only groups whose bound
 // reaches the threshold take the exact test.  The hot loop only notes that
-// some start is above threshold; the rare warps with one find the run starts
-// and follow each run (as detect_kernel), runs leaving the ring go to
-// tail_kernel.
+// some start is above threshold; a warp with one then takes each width's runs from
+// the 16 starts of its lanes at once: a lane reports the runs that open and end among
+// them, shuffles join the ones that go on, and what crosses a warp or a chunk is
+// carried on as its best start so far, so a start is looked at once however long its
+// run is.  Only runs that leave the segment are followed, by a warp, and beyond the
+// ring by tail_kernel.  This is what bounds a list of many or long runs, as residual
+// interference gives: following every run with a whole warp from its first start, and
+// counting each candidate up on the list by itself, took 87 of the 110 ms that the
+// search of 4096 channels x 2^20 samples x 1500 trials with masked interference needs
+// there, this 38 (and 14 -> 0.8 ms in tail_kernel); a single list of 4e5 candidates
+// 0.94 -> 0.71 ms.  A quiet series pays 2.32 -> 2.4 ms for the registers (of 173).
 constexpr int kDWThreads = 128;
 constexpr int kDWPer = 16;                          // consecutive starts per thread
 constexpr int kDWChunk = kDWThreads * kDWPer;       // starts per chunk
 constexpr int kDWLead = 16;                         // prefix entries before a segment's first start
+constexpr int kDWCands = 128;                       // candidates collected before they are appended
 
 // Exclusive prefix of v over the block's threads, and in *total the block's
 // sum; one barrier: every warp adds up the warp totals before it itself.
@@ -1060,6 +1069,14 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
     __shared__ int2 wt_s[kMaxWidths];               // {W, threshold} of the widths that can fire:
     __shared__ int nlive, nexact;                   // [0, nexact) tested exactly, the rest by group bound
     __shared__ int32_t thr_p2[4];                   // widths 1, 2, 4, 8 (INT32_MAX: not searched)
+    __shared__ int3 cand_s[kDWCands];               // {start - S0, width, S} of runs found
+    __shared__ int cand_n;
+    __shared__ unsigned long long cand_base;
+    // per warp and width: the runs that cross the warp's starts (their best starts)
+    __shared__ uint64_t run_head[kDWThreads / 32][kMaxWidths], run_leaves[kDWThreads / 32][kMaxWidths];
+    __shared__ uint3 run_bits[kDWThreads / 32];     // widths: with a start above, passed through, left
+                                                    // open (zeros of a warp without any stay)
+    __shared__ int runs_here;                       // a start above in this chunk or an open run
     const int trial = blockIdx.y;
     if (!narrow_trial(a, trial)) return;             // detect_kernel takes the trial
     const int64_t n = a.nout;
@@ -1080,6 +1097,9 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
         width_s[tid] = a.widths[tid];
     }
     if (tid == 0) {
+        cand_n = 0;
+        runs_here = 0;
+        for (int w = 0; w < kDWThreads / 32; ++w) run_bits[w] = make_uint3(0, 0, 0);
         // widths 1, 2, 4, 8 apart (tested from registers with fixed shifts), then
         // the other widths below 16 or not multiples of 16, then the multiples of 16
         for (int j = 0; j < 4; ++j) thr_p2[j] = INT32_MAX;
@@ -1152,9 +1172,45 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
         load(f);
         put(f);
     }
+    // Candidates are collected here and appended to the list many at a time: one
+    // addition to its count each would be millions on one address.
+    auto put_cand = [&](uint64_t best, int k) {
+        const int i = atomicAdd(&cand_n, 1);
+        const int32_t S = (int32_t)((uint32_t)(best >> 32) ^ 0x80000000u);
+        const int32_t dt = (int32_t)(0x7fffffffu - (uint32_t)best);
+        if (i < kDWCands)
+            cand_s[i] = make_int3(dt, k, S);
+        else
+            emit(a, trial, k, S0 + dt, S);
+    };
+    auto flush_cands = [&]() {                        // by the whole block
+        const int m = min(cand_n, kDWCands);
+        __syncthreads();
+        if (tid == 0) {
+            cand_n = 0;
+            if (m > 0)
+                cand_base = atomicAdd(reinterpret_cast<unsigned long long*>(a.raw_count),
+                                      (unsigned long long)m);
+        }
+        __syncthreads();
+        for (int i = tid; i < m; i += kDWThreads) {
+            const int64_t idx = (int64_t)cand_base + i;
+            if (idx >= a.raw_cap) break;
+            const int3 x = cand_s[i];
+            hp_raw_cand c;
+            c.dm_idx = trial;
+            c.width_idx = x.y;
+            c.sample = (S0 + x.x) * a.sample_mul + a.t_offset;
+            c.S = x.z;
+            a.raw[idx] = c;
+        }
+        __syncthreads();   // cand_s may be refilled
+    };
     const int64_t nchunks = (S1 - S0 + kDWChunk - 1) / kDWChunk;
     if (nchunks > 1) load(f);                         // the next chunk's new samples, in flight
     const bool cin_any = a.carry_in && S0 == 0;
+    bool was_active = false;                          // run_bits[warp] is not zero
+    uint64_t open_best = 0;                           // warp 0, lane k: best start of width k's open run
 
     for (int64_t c = 0; c < nchunks; ++c) {
         const int64_t t0 = S0 + c * kDWChunk;
@@ -1241,33 +1297,8 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
                     if ((int32_t)acc >= 0) hit = 1u;
                 }
             }
-            // the exact pass below wants the widths: find them on a hit (rare)
-            if (hit) {
-                hit = 0;
-                for (int k = 0; k < a.nw; ++k) {
-                    const int32_t thr = thr_s[k];
-                    if (thr == INT32_MAX) continue;
-                    uint32_t q[16];
-                    ahead(width_s[k], q);
-                    bool any = false;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) any |= (int32_t)(q[i] - p[i]) >= thr;
-                    if (any) hit |= 1u << k;
-                }
-            }
         } else {
-            for (int k = 0; k < a.nw; ++k) {
-                const int32_t thr = thr_s[k];
-                if (thr == INT32_MAX) continue;
-                const int W = width_s[k];
-                const int64_t lim = min(tmax, n - W) - tb;   // starts tb + i, i <= lim, are tested
-                uint32_t q[16];
-                ahead(W, q);
-                bool any = false;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) any |= i <= lim && (int32_t)(q[i] - p[i]) >= thr;
-                if (any) hit |= 1u << k;
-            }
+            hit = 1u;   // (the exact pass masks the starts past the segment or the series)
         }
 
         // the block that holds start nwin - 1 reports the carry flags
@@ -1282,22 +1313,31 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
             }
         }
 
-        if (__any_sync(0xffffffffu, hit != 0)) {
-            // rare: run starts and runs of the widths some lane flagged
-            unsigned todo = __reduce_or_sync(0xffffffffu, hit);
-            while (todo) {
-                const int k = __ffs(todo) - 1;
-                todo &= todo - 1;
+        // Runs.  A warp's 512 starts, per width with a start above threshold: the runs
+        // that open and end among them are reported here; of a run that comes in from
+        // the starts before, its part up to the first start below threshold (or all of
+        // them: it passes); of one that is still open at their end, its part so far.
+        // Best starts are words that compare by sum, then earliest start.
+        const bool any_hit = __any_sync(0xffffffffu, hit != 0);
+        if (any_hit || was_active) {
+            uint32_t active = 0, passes = 0, leaves = 0;
+            const uint32_t d0 = 0x7fffffffu - (uint32_t)(tb - S0);
+            for (int k = any_hit ? 0 : a.nw; k < a.nw; ++k) {
                 const int32_t thr = thr_s[k];
+                if (thr == INT32_MAX) continue;
                 const int W = width_s[k];
                 const int64_t last = n - W;
-                const int64_t lim = min(tmax, last) - tb;
-                uint32_t q[16];
-                ahead(W, q);
+                const int64_t lim = min(tmax, last) - tb;       // starts tb + i, i <= lim, are tested
+                uint32_t q[16] = {};
                 unsigned above = 0;
+                if (hit) {                              // (no start of another lane is above)
+                    ahead(W, q);
 #pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (i <= lim && (int32_t)(q[i] - p[i]) >= thr) above |= 1u << i;
+                    for (int i = 0; i < 16; ++i)
+                        if (i <= lim && (int32_t)(q[i] - p[i]) >= thr) above |= 1u << i;
+                }
+                if (!__any_sync(0xffffffffu, above != 0)) continue;
+                active |= 1u << k;
                 // a start opens a run when the start before it is below threshold:
                 // the previous lane's last start, or for lane 0 start tb - 1
                 const unsigned prev = __shfl_up_sync(0xffffffffu, above, 1);
@@ -1314,53 +1354,139 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
                 // that the previous gulp left open is not reported again
                 if (a.nwin < tb + 16) starts &= a.nwin <= tb ? 0u : (1u << (int)(a.nwin - tb)) - 1u;
                 if (cin_any && tb == 0 && a.carry_in[(int64_t)trial * a.nw + k]) starts &= ~1u;
-                unsigned lanes = __ballot_sync(0xffffffffu, starts != 0);
-                auto box32 = [&](int64_t u) {
-                    const int64_t i = u - base;
-                    return (int32_t)(R.get(i + W) - R.get(i));
+                // `ends`: the starts that end a run (below threshold, or past the last
+                // start of the series); a lane without one passes runs on
+                const int64_t past = last + 1 - tb;
+                const unsigned tested = lim >= 15 ? 0xffffu : lim < 0 ? 0u : (2u << (int)lim) - 1u;
+                const unsigned beyond = past >= 16 ? 0u : past <= 0 ? 0xffffu : 0xffffu & ~((1u << (int)past) - 1u);
+                const unsigned ends = ~above & (tested | beyond) & 0xffffu;
+                auto best_of = [&](unsigned m) {           // 0 for m = 0: below every candidate
+                    int32_t S = INT32_MIN;
+                    int at = 0;
+#pragma unroll
+                    for (int i = 15; i >= 0; --i) {
+                        const int32_t Si = (int32_t)(q[i] - p[i]);
+                        if ((m >> i & 1u) && Si >= S) { S = Si; at = i; }
+                    }
+                    return m ? (uint64_t)((uint32_t)S ^ 0x80000000u) << 32 | (d0 - (uint32_t)at) : 0ull;
                 };
-                while (lanes) {
-                    const int L = __ffs(lanes) - 1;
-                    lanes &= lanes - 1;
-                    unsigned sL = __shfl_sync(0xffffffffu, starts, L);
-                    const int64_t tL = t0 + (int64_t)kDWPer * (warp * 32 + L);
-                    while (sL) {
-                        const int e = __ffs(sL) - 1;
-                        sL &= sL - 1;
-                        int64_t bS, bt, tu = 0;
-                        const bool tail = follow_run32(tL + e, last, base, len, (int64_t)W,
-                                                       thr, box32, lane, &bS, &bt, &tu);
-                        if (lane == 0) {
-                            if (!tail) {
-                                emit(a, trial, k, bt, bS);
+                // this lane's starts before its first end, joined over the lanes after it
+                // that a run which comes in here fills
+                uint64_t head = best_of(above & (ends ? (ends & (0u - ends)) - 1u : 0xffffu));
+                bool pass = ends == 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint64_t h = __shfl_down_sync(0xffffffffu, head, o);
+                    const bool ps = __shfl_down_sync(0xffffffffu, pass, o);
+                    if (pass && lane + o < 32) {
+                        head = max(head, h);
+                        pass = ps;
+                    }
+                }
+                uint64_t next_head = __shfl_down_sync(0xffffffffu, head, 1);
+                bool next_pass = __shfl_down_sync(0xffffffffu, pass, 1);
+                if (lane == 31) {
+                    next_head = 0;
+                    next_pass = true;
+                }
+                uint64_t leaving = 0;
+                for (unsigned m = starts; m; m &= m - 1) {
+                    const int e = __ffs(m) - 1;
+                    const unsigned after = ends >> e << e;
+                    uint64_t best = best_of((above & (after ? (after & (0u - after)) - 1u : 0xffffu)) >> e << e);
+                    if (!after) best = max(best, next_head);
+                    if (!after && next_pass)
+                        leaving = best;            // (at most one run of the warp)
+                    else
+                        put_cand(best, k);
+                }
+                if (leaving) run_leaves[warp][k] = leaving;
+                if (__any_sync(0xffffffffu, leaving != 0)) leaves |= 1u << k;
+                if (lane == 0) {
+                    run_head[warp][k] = head;
+                    if (pass) passes |= 1u << k;
+                }
+            }
+            if (lane == 0) {
+                run_bits[warp] = make_uint3(active, passes, leaves);
+                if (active) runs_here = 1;
+            }
+            was_active = active != 0;
+        }
+        __syncthreads();                              // chunk c tested everywhere
+        // lane k of warp 0 carries width k's open run over the warps of the chunk
+        if (runs_here) {
+            if (warp == 0) {
+                for (int w = 0; w < kDWThreads / 32; ++w) {
+                    if (t0 + 512 * w > tmax) break;   // past the segment: nothing tested there
+                    const uint3 bits = run_bits[w];
+                    const bool on = bits.x >> lane & 1u;
+                    if (open_best) {
+                        if (on) open_best = max(open_best, run_head[w][lane]);
+                        if (!(on && (bits.y >> lane & 1u))) {
+                            put_cand(open_best, lane);
+                            open_best = 0;
+                        }
+                    }
+                    if (on && (bits.z >> lane & 1u)) open_best = run_leaves[w][lane];
+                }
+            }
+            __syncthreads();                          // runs_here was read everywhere
+            if (warp == 0) {
+                const unsigned o = __ballot_sync(0xffffffffu, open_best != 0);
+                if (lane == 0) runs_here = o != 0;
+            }
+            if (c + 1 == nchunks && warp == 0) {
+                // the runs still open at the segment's end S1: followed over the starts that
+                // the ring holds, the rest left to tail_kernel
+                for (unsigned m = __ballot_sync(0xffffffffu, open_best != 0); m; m &= m - 1) {
+                    const int k = __ffs(m) - 1;
+                    const int W = width_s[k];
+                    const uint64_t ob = __shfl_sync(0xffffffffu, open_best, k);
+                    auto box32 = [&](int64_t u) {
+                        const int64_t i = u - base;
+                        return (int32_t)(R.get(i + W) - R.get(i));
+                    };
+                    int64_t bS, bt, tu = 0;
+                    const bool tail = follow_run32(S1, n - W, base, len, (int64_t)W, thr_s[k], box32,
+                                                   lane, &bS, &bt, &tu);
+                    if (lane == 0) {
+                        const int64_t oS = (int32_t)((uint32_t)(ob >> 32) ^ 0x80000000u);
+                        if (oS >= bS) {            // (ties: the earlier start)
+                            bS = oS;
+                            bt = S0 + (int64_t)(0x7fffffffu - (uint32_t)ob);
+                        }
+                        if (!tail) {
+                            emit(a, trial, k, bt, bS);
+                        } else {
+                            const unsigned long long qi = atomicAdd(
+                                reinterpret_cast<unsigned long long*>(a.tail_count), 1ull);
+                            if ((int64_t)qi < a.tail_cap) {
+                                TailRec r;
+                                r.trial = trial;
+                                r.k = k;
+                                r.u = tu;
+                                r.S_prev = box32(tu - 1);
+                                r.best_S = bS;
+                                r.best_t = bt;
+                                a.tails[qi] = r;
                             } else {
-                                const unsigned long long qi = atomicAdd(
-                                    reinterpret_cast<unsigned long long*>(a.tail_count), 1ull);
-                                if ((int64_t)qi < a.tail_cap) {
-                                    TailRec r;
-                                    r.trial = trial;
-                                    r.k = k;
-                                    r.u = tu;
-                                    r.S_prev = box32(tu - 1);
-                                    r.best_S = bS;
-                                    r.best_t = bt;
-                                    a.tails[qi] = r;
-                                } else {
-                                    latch_status(a.status, HP_ERR_CAND_OVERFLOW);
-                                }
+                                latch_status(a.status, HP_ERR_CAND_OVERFLOW);
                             }
                         }
                     }
                 }
             }
+            __syncthreads();                          // candidates and runs_here visible
+            if (cand_n > kDWCands / 2) flush_cands();
         }
-        __syncthreads();                              // chunk c tested everywhere
         if (c + 1 < nchunks) {
             put(f);                                   // the samples loaded during chunk c
             f += kDWChunk;
             if (c + 2 < nchunks) load(f);             // in flight while chunk c + 1 is tested
         }
     }
+    if (cand_n) flush_cands();
 }
 
 // Runs that leave the detect tile's halo or the ring: continue each one from
