@@ -146,10 +146,10 @@ __device__ __forceinline__ void pdl_wait() {
 }
 
 template <class... P, class... A>
-cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem,
                        cudaStream_t s, const A&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

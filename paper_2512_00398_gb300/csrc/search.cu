@@ -352,18 +352,17 @@ __device__ __forceinline__ void load_chunk32(const int32_t* __restrict__ row, in
 }
 
 // Histogram of |y| per trial; also writes y = D - b (int32: |D|, |b| < 2^21)
-// for the passes after it.  A block takes kHistBlock consecutive samples of
-// one trial; each thread walks kHistSpan consecutive samples with one baseline
+// for the passes after it.  A block takes 256 spans of consecutive samples of
+// one trial; each thread walks kHistSpan of them with one baseline
 // walker (set up once, its divisions amortised over the span), kHistStep at a
 // time: every byte it loads is used, and the block's shared bins are cleared
-// and flushed once per kHistBlock samples.  Each thread reads a step before it
+// and flushed once per block.  Each thread reads a step before it
 // writes it, so Y may alias D (median mode, whose walker reads only the knots).
 constexpr int kHistThreads = 256;
-constexpr int kHistSpan = 256;                           // samples per thread
 constexpr int kHistStep = 16;                            // samples per load step
-constexpr int kHistBlock = kHistThreads * kHistSpan;     // samples per block
+__host__ __device__ constexpr int hist_block(int span) { return kHistThreads * span; }   // samples per block
 
-template <int MODE>
+template <int MODE, int kHistSpan>
 __global__ void __launch_bounds__(kHistThreads, 4) mad_hist_kernel(const int32_t* D, int64_t pitch,
                                                                 int64_t n, BaselineCtx bc, int vec,
                                                                 uint32_t* __restrict__ hist,
@@ -371,6 +370,7 @@ __global__ void __launch_bounds__(kHistThreads, 4) mad_hist_kernel(const int32_t
                                                                 int yvec) {
     __shared__ uint32_t h[kHistBins];
     __shared__ __align__(16) int4 tile[kHistThreads / 32][32 * kHistStep / 4];
+    constexpr int kHistBlock = hist_block(kHistSpan);
     const int trial = blockIdx.y;
     for (int i = threadIdx.x; i < kHistBins; i += blockDim.x) h[i] = 0;
     __syncthreads();
@@ -498,158 +498,6 @@ __global__ void __launch_bounds__(kHistThreads, 4) mad_hist_kernel(const int32_t
         if (h[i]) atomicAdd(&g[i], h[i]);
 }
 
-// Block-wide search of the bin holding rank k (0-based) in a histogram of
-// `bins` counts.  Returns the bin and the count of all earlier bins.
-__device__ void find_rank_bin(const uint32_t* __restrict__ hrow, int bins, int64_t k, int* bin_out,
-                              int64_t* before_out) {
-    __shared__ int64_t part[1024];
-    __shared__ int s_bin;
-    __shared__ int64_t s_before;
-    const int per = (bins + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * per;
-    int64_t mine = 0;
-    for (int b = b0; b < min(bins, b0 + per); ++b) mine += hrow[b];
-    part[threadIdx.x] = mine;
-    if (threadIdx.x == 0) { s_bin = -1; s_before = 0; }
-    __syncthreads();
-    for (int o = 1; o < (int)blockDim.x; o <<= 1) {   // inclusive Hillis-Steele scan
-        const int64_t v = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    const int64_t incl = part[threadIdx.x];
-    const int64_t excl = incl - mine;
-    if (excl <= k && k < incl) {
-        int64_t c = excl;
-        for (int b = b0; b < min(bins, b0 + per); ++b) {
-            if (k < c + hrow[b]) { s_bin = b; s_before = c; break; }
-            c += hrow[b];
-        }
-    }
-    __syncthreads();
-    *bin_out = s_bin;
-    *before_out = s_before;
-}
-
-__global__ void __launch_bounds__(1024) mad_select_kernel(uint32_t* __restrict__ hist, int64_t n,
-                                                          int32_t* __restrict__ bucket,
-                                                          int64_t* __restrict__ rank,
-                                                          int64_t* __restrict__ mad,
-                                                          int64_t* __restrict__ ybound) {
-    const int trial = blockIdx.x;
-    uint32_t* hrow = hist + (int64_t)trial * kHistBins;
-    const int64_t k = (n - 1) / 2;
-    if (ybound) {
-        // an upper bound of max |y| from the highest non-empty bin: exact below
-        // kHistFine, the top of a coarse bin above, none for the last coarse bin
-        __shared__ int s_top;
-        if (threadIdx.x == 0) s_top = -1;
-        __syncthreads();
-        int top = -1;
-        for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
-            if (hrow[b]) top = b;
-        if (top >= 0) atomicMax(&s_top, top);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int t = s_top;
-            ybound[trial] = t < 0 ? 0
-                          : t < kHistFine ? (int64_t)t
-                          : t == kHistBins - 1 ? -1
-                          : ((int64_t)(t - kHistFine + 1) << 12) - 1;
-        }
-    }
-    int bin;
-    int64_t before;
-    find_rank_bin(hrow, kHistBins, k, &bin, &before);
-    if (threadIdx.x == 0) {
-        if (bin < kHistFine) {
-            mad[trial] = bin;
-            bucket[trial] = -1;
-        } else {
-            bucket[trial] = bin - kHistFine;
-            rank[trial] = k - before;
-        }
-    }
-    __syncthreads();
-    if (bin >= kHistFine)   // reuse the row for the refinement histogram
-        for (int i = threadIdx.x; i < kHistFine; i += blockDim.x) hrow[i] = 0;
-}
-
-__global__ void __launch_bounds__(256) mad_refine_hist_kernel(const int32_t* __restrict__ Y,
-                                                              int64_t ypitch, int64_t n, int yvec,
-                                                              const int32_t* __restrict__ bucket,
-                                                              uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[kHistFine];
-    const int trial = blockIdx.y;
-    const int32_t B = bucket[trial];
-    if (B < 0) return;
-    for (int i = threadIdx.x; i < kHistFine; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    const int32_t* yrow = Y + (int64_t)trial * ypitch;
-    const int64_t t_begin = (int64_t)blockIdx.x * kHistChunk + threadIdx.x * 32;
-    const int64_t t_end = min(n, t_begin + 32);
-    if (t_begin < t_end) {
-        int32_t v[32];
-        load_chunk32(yrow, t_begin, t_end, yvec != 0, v);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            if (t_begin + q < t_end) {
-                const int64_t y = v[q] < 0 ? -(int64_t)v[q] : (int64_t)v[q];
-                if ((y >> 12) == B) atomicAdd(&h[y & 4095], 1u);
-            }
-        }
-    }
-    __syncthreads();
-    uint32_t* g = hist + (int64_t)trial * kHistBins;
-    for (int i = threadIdx.x; i < kHistFine; i += blockDim.x)
-        if (h[i]) atomicAdd(&g[i], h[i]);
-}
-
-__global__ void __launch_bounds__(1024) mad_refine_select_kernel(
-    const uint32_t* __restrict__ hist, const int32_t* __restrict__ bucket,
-    const int64_t* __restrict__ rank, int64_t* __restrict__ mad) {
-    const int trial = blockIdx.x;
-    const int32_t B = bucket[trial];
-    if (B < 0) return;
-    int bin;
-    int64_t before;
-    find_rank_bin(hist + (int64_t)trial * kHistBins, kHistFine, rank[trial], &bin, &before);
-    if (threadIdx.x == 0) mad[trial] = ((int64_t)B << 12) + bin;
-}
-
-// sigma and the integer thresholds ceil(thr * sigma * sqrt(W)) per (trial, width)
-__global__ void sigma_kernel(const int64_t* __restrict__ mad, int ndm,
-                             const int32_t* __restrict__ widths, int nw, float thr,
-                             double* __restrict__ sigma, int64_t* __restrict__ tint) {
-    const int trial = blockIdx.x * blockDim.x + threadIdx.x;
-    if (trial >= ndm) return;
-    const double sg = __dmul_rn(kMadToSigma, (double)mad[trial]);
-    sigma[trial] = sg;
-    for (int k = 0; k < nw; ++k) {
-        int64_t v = kNever;
-        if (sg > 0.0) {
-            const double lim = __dmul_rn(__dmul_rn((double)thr, sg), __dsqrt_rn((double)widths[k]));
-            v = (int64_t)ceil(lim);
-        }
-        tint[(int64_t)trial * nw + k] = v;
-    }
-}
-
-// ------------------------------------------------------------ detection
-constexpr int kDetectThreads = 256;
-constexpr int kDetectPer = kDetectTile / kDetectThreads;   // starts per thread
-
-// Every boxcar sum of this trial fits int32 with room to spare: its |y| bound
-// times (the widest boxcar + 32) stays below 2^31 - 1 (the 32-bit detection's
-// group bound adds two 15-sample partial sums to a boxcar sum).
-__device__ __forceinline__ bool narrow_trial(const SearchArgs& a, int trial) {
-    if (!a.ybound) return false;
-    const int64_t yb = a.ybound[trial];
-    return yb >= 0 && yb * (a.ybound_w + 32) < (int64_t)INT32_MAX;
-}
-
-
 __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* warp_tot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int64_t x = v;
@@ -672,6 +520,142 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* warp
     __syncthreads();
     return x - v + (warp > 0 ? warp_tot[warp - 1] : 0);
 }
+
+// Block-wide search of the bin holding rank k (0-based) in a histogram of
+// `bins` counts.  Returns the bin and the count of all earlier bins.
+__device__ void find_rank_bin(const uint32_t* hrow, int bins, int64_t k, int* bin_out,
+                              int64_t* before_out) {
+    __shared__ int64_t warp_tot[32];
+    __shared__ int s_bin;
+    __shared__ int64_t s_before;
+    const int per = (bins + blockDim.x - 1) / blockDim.x;
+    const int b0 = threadIdx.x * per, b1 = min(bins, b0 + per);
+    int64_t mine = 0;
+    for (int b = b0; b < b1; ++b) mine += hrow[b];
+    if (threadIdx.x == 0) { s_bin = -1; s_before = 0; }
+    const int64_t excl = block_exclusive_scan(mine, warp_tot);   // (synchronises)
+    if (excl <= k && k < excl + mine) {
+        int64_t c = excl;
+        for (int b = b0; b < b1; ++b) {
+            if (k < c + hrow[b]) { s_bin = b; s_before = c; break; }
+            c += hrow[b];
+        }
+    }
+    __syncthreads();
+    *bin_out = s_bin;
+    *before_out = s_before;
+}
+
+// sigma = 1.4826.. x MAD and the integer thresholds ceil(thr * sigma * sqrt(W)) of a
+// trial's widths, by the block whose select found the MAD (a kernel of its own, a thread
+// per trial, took 6 to 10 us)
+__device__ __forceinline__ void write_thresholds(const SearchArgs& a, int trial, int64_t mad) {
+    const double sg = __dmul_rn(kMadToSigma, (double)mad);
+    if (threadIdx.x == 0) {
+        a.mad[trial] = mad;
+        a.sigma[trial] = sg;
+    }
+    for (int k = threadIdx.x; k < a.nw; k += blockDim.x) {
+        int64_t v = kNever;
+        if (sg > 0.0) {
+            const double lim = __dmul_rn(__dmul_rn((double)a.thr, sg), __dsqrt_rn((double)a.widths[k]));
+            v = (int64_t)ceil(lim);
+        }
+        a.tint[(int64_t)trial * a.nw + k] = v;
+    }
+}
+
+__global__ void __launch_bounds__(1024) mad_select_kernel(const __grid_constant__ SearchArgs a) {
+    pdl_wait();
+    const int trial = blockIdx.x;
+    uint32_t* hrow = a.hist + (int64_t)trial * kHistBins;
+    const int64_t k = (a.nout - 1) / 2;
+    if (a.ybound) {
+        // an upper bound of max |y| from the highest non-empty bin: exact below
+        // kHistFine, the top of a coarse bin above, none for the last coarse bin
+        __shared__ int s_top;
+        if (threadIdx.x == 0) s_top = -1;
+        __syncthreads();
+        int top = -1;
+        for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
+            if (hrow[b]) top = b;
+        if (top >= 0) atomicMax(&s_top, top);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const int t = s_top;
+            a.ybound[trial] = t < 0 ? 0
+                          : t < kHistFine ? (int64_t)t
+                          : t == kHistBins - 1 ? -1
+                          : ((int64_t)(t - kHistFine + 1) << 12) - 1;
+        }
+    }
+    int bin;
+    int64_t before;
+    find_rank_bin(hrow, kHistBins, k, &bin, &before);
+    if (threadIdx.x == 0) {
+        a.refine_bucket[trial] = bin < kHistFine ? -1 : bin - kHistFine;
+        a.refine_rank[trial] = k - before;
+    }
+    if (bin < kHistFine)
+        write_thresholds(a, trial, bin);
+    else                    // reuse the row for the refinement histogram
+        for (int i = threadIdx.x; i < kHistFine; i += blockDim.x) hrow[i] = 0;
+}
+
+__global__ void __launch_bounds__(256) mad_refine_hist_kernel(const __grid_constant__ SearchArgs a,
+                                                              int yvec) {
+    __shared__ uint32_t h[kHistFine];
+    pdl_wait();
+    const int trial = blockIdx.y;
+    const int32_t B = a.refine_bucket[trial];
+    if (B < 0) return;
+    const int64_t n = a.nout;
+    for (int i = threadIdx.x; i < kHistFine; i += blockDim.x) h[i] = 0;
+    __syncthreads();
+    const int32_t* yrow = a.Y + (int64_t)trial * a.ypitch;
+    const int64_t t_begin = (int64_t)blockIdx.x * kHistChunk + threadIdx.x * 32;
+    const int64_t t_end = min(n, t_begin + 32);
+    if (t_begin < t_end) {
+        int32_t v[32];
+        load_chunk32(yrow, t_begin, t_end, yvec != 0, v);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+            if (t_begin + q < t_end) {
+                const int64_t y = v[q] < 0 ? -(int64_t)v[q] : (int64_t)v[q];
+                if ((y >> 12) == B) atomicAdd(&h[y & 4095], 1u);
+            }
+        }
+    }
+    __syncthreads();
+    uint32_t* g = a.hist + (int64_t)trial * kHistBins;
+    for (int i = threadIdx.x; i < kHistFine; i += blockDim.x)
+        if (h[i]) atomicAdd(&g[i], h[i]);
+}
+
+__global__ void __launch_bounds__(1024) mad_refine_select_kernel(const __grid_constant__ SearchArgs a) {
+    pdl_wait();
+    const int trial = blockIdx.x;
+    const int32_t B = a.refine_bucket[trial];
+    if (B < 0) return;
+    int bin;
+    int64_t before;
+    find_rank_bin(a.hist + (int64_t)trial * kHistBins, kHistFine, a.refine_rank[trial], &bin, &before);
+    write_thresholds(a, trial, ((int64_t)B << 12) + bin);
+}
+
+// ------------------------------------------------------------ detection
+constexpr int kDetectThreads = 256;
+constexpr int kDetectPer = kDetectTile / kDetectThreads;   // starts per thread
+
+// Every boxcar sum of this trial fits int32 with room to spare: its |y| bound
+// times (the widest boxcar + 32) stays below 2^31 - 1 (the 32-bit detection's
+// group bound adds two 15-sample partial sums to a boxcar sum).
+__device__ __forceinline__ bool narrow_trial(const SearchArgs& a, int trial) {
+    if (!a.ybound) return false;
+    const int64_t yb = a.ybound[trial];
+    return yb >= 0 && yb * (a.ybound_w + 32) < (int64_t)INT32_MAX;
+}
+
 
 __device__ __forceinline__ void emit(const SearchArgs& a, int trial, int k, int64_t t, int64_t S) {
     const unsigned long long idx = atomicAdd(reinterpret_cast<unsigned long long*>(a.raw_count), 1ull);
@@ -955,6 +939,7 @@ __device__ void detect_tile(const SearchArgs& a, int trial, int64_t tile) {
 // trials this kernel takes are rare, and the others leave at once.
 constexpr int kDetectBlocksPerTrial = 8;
 __global__ void __launch_bounds__(kDetectThreads) detect_kernel(const __grid_constant__ SearchArgs a) {
+    pdl_wait();
     const int trial = blockIdx.y;
     if (narrow_trial(a, trial)) return;   // detect32_kernel takes the trial
     const int64_t ntiles = (a.nout + kDetectTile - 1) / kDetectTile;
@@ -1077,6 +1062,7 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
     __shared__ uint3 run_bits[kDWThreads / 32];     // widths: with a start above, passed through, left
                                                     // open (zeros of a warp without any stay)
     __shared__ int runs_here;                       // a start above in this chunk or an open run
+    pdl_wait();
     const int trial = blockIdx.y;
     if (!narrow_trial(a, trial)) return;             // detect_kernel takes the trial
     const int64_t n = a.nout;
@@ -1499,6 +1485,7 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
 constexpr int kTailPer = 4;
 
 __global__ void tail_kernel(const __grid_constant__ SearchArgs a) {
+    pdl_wait();
     const int64_t cnt = min(*a.tail_count, a.tail_cap);
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -1853,8 +1840,7 @@ cudaError_t launch_detect(const SearchArgs& a, cudaStream_t s, int64_t* nlaunch)
     const dim3 dgrid((unsigned)std::min<int64_t>(ceil_div(a.nout, kDetectTile), kDetectBlocksPerTrial),
                      a.ndm);
     ++*nlaunch;
-    detect_kernel<<<dgrid, kDetectThreads, smem, s>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(detect_kernel, dgrid, kDetectThreads, smem, s, a)) != cudaSuccess) return e;
     // the trials whose boxcar sums all fit int32 (nearly all): a block per
     // segment of a trial, about 10 000 blocks, at least 4 chunks per segment
     const int64_t f0 = ceil_div(kDWLead + kDWChunk + (int64_t)a.wmax + 1, kDWChunk) * kDWChunk;
@@ -1870,11 +1856,10 @@ cudaError_t launch_detect(const SearchArgs& a, cudaStream_t s, int64_t* nlaunch)
     const int64_t seg = ceil_div(chunks, nseg) * kDWChunk;
     const dim3 dgrid32((unsigned)ceil_div(a.nout, seg), a.ndm);
     ++*nlaunch;
-    detect32_kernel<<<dgrid32, kDWThreads, smem32, s>>>(a, seg, ring);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(detect32_kernel, dgrid32, kDWThreads, smem32, s, a, seg, ring)) != cudaSuccess)
+        return e;
     ++*nlaunch;
-    tail_kernel<<<2048, 128, 0, s>>>(a);   // a warp per run; idle warps leave at once
-    return cudaGetLastError();
+    return launch_pdl(tail_kernel, dim3(2048), 128, 0, s, a);   // a warp per run; idle warps leave at once
 }
 
 template <int MODE>
@@ -1887,23 +1872,33 @@ cudaError_t launch_walkers(const SearchArgs& a, const BaselineCtx& bc, cudaStrea
     const int vec = ((a.pitch & 3) == 0) && (((uintptr_t)a.D & 15u) == 0);
     const int yvec = ((a.ypitch & 3) == 0) && (((uintptr_t)a.Y & 15u) == 0);
     ++*nlaunch;
-    mad_hist_kernel<MODE><<<dim3((unsigned)ceil_div(n, kHistBlock), ndm), kHistThreads, 0, s>>>(
-        a.D, a.pitch, n, bc, vec, a.hist, a.Y, a.ypitch, yvec);
+    // The span of a thread: long ones walk fastest, but a series' last block is padded
+    // to 256 spans and few blocks leave SMs idle.  Detection of given series, spans of
+    // 256 / 64 / 32 samples, us (median baseline; the mean's, whose walkers cost more to
+    // set up and to step, fall alike):
+    //    100 x  32000   95 /  75 /  70    700 x  50000  307 / 284 / 292
+    //    200 x  50000  132 / 113 / 116    300 x 200000  399 / 381 / 398
+    //    300 x  65536  148 / 153 / 166   2000 x   9000  346 / 242 / 252
+    auto blocks = [&](int span) { return ceil_div(n, hist_block(span)) * ndm; };
+    auto hist = [&](auto span) {
+        constexpr int kSpan = decltype(span)::value;
+        mad_hist_kernel<MODE, kSpan><<<dim3((unsigned)ceil_div(n, hist_block(kSpan)), ndm), kHistThreads, 0, s>>>(
+            a.D, a.pitch, n, bc, vec, a.hist, a.Y, a.ypitch, yvec);
+    };
+    const int64_t padding = ceil_div(n, hist_block(256)) * hist_block(256) - n;
+    if (padding <= n / 8 && blocks(256) >= 300)
+        hist(std::integral_constant<int, 256>{});
+    else if (blocks(64) >= 600)                           // four blocks an SM
+        hist(std::integral_constant<int, 64>{});
+    else
+        hist(std::integral_constant<int, 32>{});
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ++*nlaunch;
-    mad_select_kernel<<<ndm, 1024, 0, s>>>(a.hist, n, a.refine_bucket, a.refine_rank, a.mad,
-                                           a.ybound);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(mad_select_kernel, dim3(ndm), 1024, 0, s, a)) != cudaSuccess) return e;
     ++*nlaunch;
-    mad_refine_hist_kernel<<<hgrid, 256, 0, s>>>(a.Y, a.ypitch, n, yvec, a.refine_bucket, a.hist);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(mad_refine_hist_kernel, hgrid, 256, 0, s, a, yvec)) != cudaSuccess) return e;
     ++*nlaunch;
-    mad_refine_select_kernel<<<ndm, 1024, 0, s>>>(a.hist, a.refine_bucket, a.refine_rank, a.mad);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    ++*nlaunch;
-    sigma_kernel<<<(unsigned)ceil_div(ndm, 128), 128, 0, s>>>(a.mad, ndm, a.widths, a.nw, a.thr,
-                                                              a.sigma, a.tint);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(mad_refine_select_kernel, dim3(ndm), 1024, 0, s, a)) != cudaSuccess) return e;
     if (a.stats_only) return cudaSuccess;
     if (a.width_sigma && (e = launch_width_sigma(a, s, nlaunch)) != cudaSuccess) return e;
     if (a.ndec > 0) {
