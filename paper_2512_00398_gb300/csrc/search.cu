@@ -989,6 +989,7 @@ constexpr int kDWCands = 128;                       // candidates collected befo
 
 // Exclusive prefix of v over the block's threads, and in *total the block's
 // sum; one barrier: every warp adds up the warp totals before it itself.
+template <int kThreads>
 __device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t* warp_tot,
                                                            uint32_t* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1002,7 +1003,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t*
     __syncthreads();
     uint32_t before = 0, all = 0;
 #pragma unroll
-    for (int i = 0; i < kDWThreads / 32; ++i) {
+    for (int i = 0; i < kThreads / 32; ++i) {
         const uint32_t t = warp_tot[i];
         before += i < warp ? t : 0u;
         all += t;
@@ -1141,7 +1142,7 @@ __global__ void __launch_bounds__(kDWThreads) detect32_kernel(const __grid_const
             mn = __vimin3_s32(mn, x0, x1);
         }
         uint32_t chunk_total;
-        const uint32_t off = carry + block_exclusive_scan32(run, warp_tot, &chunk_total);
+        const uint32_t off = carry + block_exclusive_scan32<kDWThreads>(run, warp_tot, &chunk_total);
 #pragma unroll
         for (int e = 0; e < 16; ++e) ex[e] += off;
         const int pos = (int)((f + kDWPer * tid) & R.mask);
@@ -1546,8 +1547,8 @@ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // ------------------------------------------------- per-width sigmas
 // The lower median of |S_k(t)| over the starts 0 <= t <= n - W_k of every
 // (trial, width), exact, by radix selection (WsigState).  Each histogram
-// pass rebuilds the boxcar sums of a tile of up to 16384 starts (one block of
-// 1024 threads) from a prefix of y over the tile and its halo in
+// pass rebuilds the boxcar sums of a tile of starts (15360, or up to 16384 where
+// sums need 64 bits) from a prefix of y over the tile and its halo in
 // shared memory and counts one digit of every value still in the running,
 // per width into one shared histogram.  The first pass counts v >> s0 below
 // 4096 (and v >> (s0 + 12) above, up to 4095), with s0 chosen from the
@@ -1598,126 +1599,260 @@ __global__ void __launch_bounds__(kWsigThreads) wsig_hist_kernel(const __grid_co
     __shared__ int64_t warp_max[32];
     __shared__ int bin_lo, bin_hi;
     const int trial = blockIdx.y;
+    if (narrow_trial(a, trial)) return;                   // wsig_hist32_kernel takes the trial
     const WsigState* st = a.wstate + (int64_t)trial * a.nw;
     bool any = false;
     for (int k = 0; k < a.nw; ++k) any = any || st[k].level == level;
     if (!any) return;                                     // the whole block
     const int64_t n = a.nout;
-    const int64_t t0 = (int64_t)blockIdx.x * tile;
-    const int len = (int)min((int64_t)tile + a.wmax - 1, n - t0);
-    const int32_t* yrow = a.Y + (int64_t)trial * a.ypitch + t0;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < len; i += blockDim.x) P[i + 1] = (int64_t)yrow[i];
-    __syncthreads();
-    const int per = ((len + (int)blockDim.x - 1) / (int)blockDim.x) | 1;
-    const int i0 = min(len, tid * per), i1 = min(len, i0 + per);
-    int64_t local = 0, ymax = 0;
-    for (int i = i0; i < i1; ++i) {
-        const int64_t y = P[i + 1];
-        local += y;
-        ymax = max(ymax, y < 0 ? -y : y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ymax = max(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
-    if (lane == 0) warp_max[warp] = ymax;
-    int64_t run = block_exclusive_scan(local, warp_tot);  // (synchronises)
-    for (int i = i0; i < i1; ++i) {
-        run += P[i + 1];
-        P[i + 1] = run;
-    }
-    if (tid == 0) {
-        P[0] = 0;
-        bin_lo = kWsigBins;
-        bin_hi = -1;
-    }
-    __syncthreads();
-    int64_t tile_max = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tile_max = max(tile_max, warp_max[w]);
-    // every boxcar sum of this tile fits int32: wrapped 32-bit differences of
-    // the prefix's low words are exact
-    const bool narrow = tile_max * (int64_t)a.wmax < (int64_t)INT32_MAX;
-    const uint32_t* P32 = reinterpret_cast<const uint32_t*>(P);   // low word of P[i]: P32[2 i]
-    for (int i = tid; i < kWsigBins; i += blockDim.x) h[i] = 0;
-    for (int k = 0; k < a.nw; ++k) {
-        const WsigState sk = st[k];
-        if (sk.level != level) continue;                  // uniform over the block
+    for (int64_t tl = blockIdx.x; tl * tile < n; tl += gridDim.x) {
+        const int64_t t0 = tl * tile;
+        const int len = (int)min((int64_t)tile + a.wmax - 1, n - t0);
+        const int32_t* yrow = a.Y + (int64_t)trial * a.ypitch + t0;
+        const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+        for (int i = tid; i < len; i += blockDim.x) P[i + 1] = (int64_t)yrow[i];
         __syncthreads();
-        const int W = a.widths[k];
-        const int t_end = (int)min((int64_t)tile, n - W + 1 - t0);   // starts of this tile
-        int lo = kWsigBins, hi = -1;
-        bool big = false;
-        if (narrow) {
-            // every |S| < 2^31: the digit in 32-bit arithmetic (a shift of 31
-            // or more leaves 0)
-            const int sh = sk.shift;
-            const uint32_t s1 = (uint32_t)min(sh, 31), s2 = (uint32_t)min(sh + 12, 31);
-            const bool z1 = sh >= 31, z2 = sh + 12 >= 31;
-            const int d = min(12, sh);
-            const uint32_t s3 = (uint32_t)min(sh - d, 31);
-            const bool z3 = sh - d >= 31;
-            const uint32_t mask = (1u << d) - 1u;
-            const bool reach = sk.prefix < ((int64_t)1 << 31);   // a 31-bit value can match
-            const uint32_t pre = (uint32_t)sk.prefix;
-            if (level == 1) {
-                for (int t = tid; t < t_end; t += blockDim.x) {
-                    const int32_t S = (int32_t)(P32[2 * (t + W)] - P32[2 * t]);
-                    const uint32_t v = S < 0 ? 0u - (uint32_t)S : (uint32_t)S;
-                    const uint32_t k1 = z1 ? 0u : v >> s1;
-                    const int b = k1 < 4096u ? (int)k1 : 4096 + (int)min(z2 ? 0u : v >> s2, 4095u);
-                    atomicAdd(&h[b], 1u);
-                    lo = min(lo, b);
-                    hi = max(hi, b);
+        const int per = ((len + (int)blockDim.x - 1) / (int)blockDim.x) | 1;
+        const int i0 = min(len, tid * per), i1 = min(len, i0 + per);
+        int64_t local = 0, ymax = 0;
+        for (int i = i0; i < i1; ++i) {
+            const int64_t y = P[i + 1];
+            local += y;
+            ymax = max(ymax, y < 0 ? -y : y);
+        }
+    #pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ymax = max(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
+        if (lane == 0) warp_max[warp] = ymax;
+        int64_t run = block_exclusive_scan(local, warp_tot);  // (synchronises)
+        for (int i = i0; i < i1; ++i) {
+            run += P[i + 1];
+            P[i + 1] = run;
+        }
+        if (tid == 0) {
+            P[0] = 0;
+            bin_lo = kWsigBins;
+            bin_hi = -1;
+        }
+        __syncthreads();
+        int64_t tile_max = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tile_max = max(tile_max, warp_max[w]);
+        // every boxcar sum of this tile fits int32: wrapped 32-bit differences of
+        // the prefix's low words are exact
+        const bool narrow = tile_max * (int64_t)a.wmax < (int64_t)INT32_MAX;
+        const uint32_t* P32 = reinterpret_cast<const uint32_t*>(P);   // low word of P[i]: P32[2 i]
+        for (int i = tid; i < kWsigBins; i += blockDim.x) h[i] = 0;
+        for (int k = 0; k < a.nw; ++k) {
+            const WsigState sk = st[k];
+            if (sk.level != level) continue;                  // uniform over the block
+            __syncthreads();
+            const int W = a.widths[k];
+            const int t_end = (int)min((int64_t)tile, n - W + 1 - t0);   // starts of this tile
+            int lo = kWsigBins, hi = -1;
+            bool big = false;
+            if (narrow) {
+                // every |S| < 2^31: the digit in 32-bit arithmetic (a shift of 31
+                // or more leaves 0)
+                const int sh = sk.shift;
+                const uint32_t s1 = (uint32_t)min(sh, 31), s2 = (uint32_t)min(sh + 12, 31);
+                const bool z1 = sh >= 31, z2 = sh + 12 >= 31;
+                const int d = min(12, sh);
+                const uint32_t s3 = (uint32_t)min(sh - d, 31);
+                const bool z3 = sh - d >= 31;
+                const uint32_t mask = (1u << d) - 1u;
+                const bool reach = sk.prefix < ((int64_t)1 << 31);   // a 31-bit value can match
+                const uint32_t pre = (uint32_t)sk.prefix;
+                if (level == 1) {
+                    for (int t = tid; t < t_end; t += blockDim.x) {
+                        const int32_t S = (int32_t)(P32[2 * (t + W)] - P32[2 * t]);
+                        const uint32_t v = S < 0 ? 0u - (uint32_t)S : (uint32_t)S;
+                        const uint32_t k1 = z1 ? 0u : v >> s1;
+                        const int b = k1 < 4096u ? (int)k1 : 4096 + (int)min(z2 ? 0u : v >> s2, 4095u);
+                        atomicAdd(&h[b], 1u);
+                        lo = min(lo, b);
+                        hi = max(hi, b);
+                    }
+                } else if (reach) {
+                    for (int t = tid; t < t_end; t += blockDim.x) {
+                        const int32_t S = (int32_t)(P32[2 * (t + W)] - P32[2 * t]);
+                        const uint32_t v = S < 0 ? 0u - (uint32_t)S : (uint32_t)S;
+                        if ((z1 ? 0u : v >> s1) == pre) {
+                            const int b = (int)((z3 ? 0u : v >> s3) & mask);
+                            atomicAdd(&h[b], 1u);
+                            lo = min(lo, b);
+                            hi = max(hi, b);
+                        }
+                    }
                 }
-            } else if (reach) {
+            } else {
                 for (int t = tid; t < t_end; t += blockDim.x) {
-                    const int32_t S = (int32_t)(P32[2 * (t + W)] - P32[2 * t]);
-                    const uint32_t v = S < 0 ? 0u - (uint32_t)S : (uint32_t)S;
-                    if ((z1 ? 0u : v >> s1) == pre) {
-                        const int b = (int)((z3 ? 0u : v >> s3) & mask);
+                    const int64_t S = P[t + W] - P[t];
+                    const uint64_t v = S < 0 ? (uint64_t)(-S) : (uint64_t)S;
+                    big = big || v >= ((uint64_t)1 << kWsigTop);
+                    const int b = wsig_bin(sk, v);
+                    if (b >= 0) {
                         atomicAdd(&h[b], 1u);
                         lo = min(lo, b);
                         hi = max(hi, b);
                     }
                 }
             }
-        } else {
-            for (int t = tid; t < t_end; t += blockDim.x) {
-                const int64_t S = P[t + W] - P[t];
-                const uint64_t v = S < 0 ? (uint64_t)(-S) : (uint64_t)S;
-                big = big || v >= ((uint64_t)1 << kWsigTop);
-                const int b = wsig_bin(sk, v);
-                if (b >= 0) {
-                    atomicAdd(&h[b], 1u);
-                    lo = min(lo, b);
-                    hi = max(hi, b);
+            if (big) latch_status(a.status, HP_ERR_INVALID_ARG);   // |S| beyond the 36-bit range
+    #pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            }
+            if (lane == 0 && hi >= 0) {
+                atomicMin(&bin_lo, lo);
+                atomicMax(&bin_hi, hi);
+            }
+            __syncthreads();
+            const int b0 = bin_lo, b1 = bin_hi;
+            __syncthreads();                                  // every thread has read the range
+            if (tid == 0) {
+                bin_lo = kWsigBins;
+                bin_hi = -1;
+            }
+            // flush the touched bins and clear them for the next width
+            uint32_t* g = a.whist + ((int64_t)trial * a.nw + k) * kWsigBins;
+            for (int i = b0 + tid; i <= b1; i += blockDim.x) {
+                const uint32_t c = h[i];
+                if (c) {
+                    atomicAdd(&g[i], c);
+                    h[i] = 0;
                 }
             }
         }
-        if (big) latch_status(a.status, HP_ERR_INVALID_ARG);   // |S| beyond the 36-bit range
+        __syncthreads();                                  // P is rebuilt for the next tile
+    }
+}
+
+// The same for the trials whose every boxcar sum fits int32 (nearly all), as
+// detect32_kernel holds them: the tile's prefix as wrapping 32-bit sums, 16 consecutive
+// starts per thread, read 16 bytes at a time.  What bounds it is shared memory: per warp
+// and 512 starts 32 wavefronts of loads and, in the first pass, 16 counting
+// instructions of about 3.5 (random banks); an int64 prefix read one start at a time took
+// 128 for the loads.  15360 starts and the halo of a 4096-sample boxcar
+// leave room for two blocks an SM, so that one counts while the other builds its prefix
+// or adds its counts to the global ones.
+// 750 trials x 2^18 samples, 13 widths: first pass 3.33 -> 2.04 ms, second 2.17 -> 0.93,
+// the two that nearly every trial leaves at once 0.17 -> 0.08 each (both kernels; the
+// blocks without work were most of it, so these take kWsigBlocksPerTrial).
+constexpr int kW32Threads = 480;
+constexpr int kW32Tile = 2 * 16 * kW32Threads;            // starts per tile
+constexpr int kWsigBlocksPerTrial = 8;                    // where few trials have work
+
+__global__ void __launch_bounds__(kW32Threads, 2) wsig_hist32_kernel(const __grid_constant__ SearchArgs a,
+                                                                     int level, int entries) {
+    extern __shared__ __align__(16) uint32_t ring_mem[];  // the prefix, then the counts
+    __shared__ uint32_t warp_tot[32];
+    const int trial = blockIdx.y;
+    if (!narrow_trial(a, trial)) return;                  // wsig_hist_kernel takes the trial
+    const WsigState* st = a.wstate + (int64_t)trial * a.nw;
+    bool any = false;
+    for (int k = 0; k < a.nw; ++k) any = any || st[k].level == level;
+    if (!any) return;                                     // the whole block
+    const int64_t n = a.nout;
+    const int32_t* yrow = a.Y + (int64_t)trial * a.ypitch;
+    const bool vec = ((a.ypitch & 3) | ((uintptr_t)a.Y & 15u)) == 0;
+    const int tid = threadIdx.x;
+    uint32_t* h = ring_mem + entries;
+    const Ring R{ring_mem, INT_MAX};                             // (no wrap: the tile is held whole)
+    for (int i = tid; i < kWsigBins; i += kW32Threads) h[i] = 0;
+    for (int64_t tl = blockIdx.x; tl * kW32Tile < n; tl += gridDim.x) {
+        const int64_t t0 = tl * kW32Tile;
+        // entry i: the sum of y over samples [t0, t0 + i)
+        uint32_t carry = 0;
+        for (int f = 0; f < entries; f += 16 * kW32Threads) {
+            const int64_t s0 = t0 + f + 16 * tid;
+            uint32_t v[16];
+            if (vec && s0 + 16 <= n) {
+                const int4* q = reinterpret_cast<const int4*>(yrow + s0);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-        }
-        if (lane == 0 && hi >= 0) {
-            atomicMin(&bin_lo, lo);
-            atomicMax(&bin_hi, hi);
-        }
-        __syncthreads();
-        const int b0 = bin_lo, b1 = bin_hi;
-        __syncthreads();                                  // every thread has read the range
-        if (tid == 0) {
-            bin_lo = kWsigBins;
-            bin_hi = -1;
-        }
-        // flush the touched bins and clear them for the next width
-        uint32_t* g = a.whist + ((int64_t)trial * a.nw + k) * kWsigBins;
-        for (int i = b0 + tid; i <= b1; i += blockDim.x) {
-            const uint32_t c = h[i];
-            if (c) {
-                atomicAdd(&g[i], c);
-                h[i] = 0;
+                for (int c = 0; c < 4; ++c) {
+                    const int4 x = __ldg(q + c);
+                    v[4 * c] = x.x; v[4 * c + 1] = x.y; v[4 * c + 2] = x.z; v[4 * c + 3] = x.w;
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) v[e] = s0 + e < n ? (uint32_t)__ldg(yrow + s0 + e) : 0u;
             }
+            uint32_t run = 0, total;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const uint32_t y = v[e];
+                v[e] = run;
+                run += y;
+            }
+            const uint32_t off = carry + block_exclusive_scan32<kW32Threads>(run, warp_tot, &total);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] += off;
+            if (f + 16 * tid < entries) R.put16(f + 16 * tid, v);
+            carry += total;
+            __syncthreads();                              // warp_tot is free again
+        }
+        for (int k = 0; k < a.nw; ++k) {
+            const WsigState sk = st[k];
+            if (sk.level != level) continue;              // uniform over the block
+            const int W = a.widths[k];
+            const int t_end = (int)min((int64_t)kW32Tile, n - W + 1 - t0);   // starts of this tile
+            // digits of values below 2^31: a shift of 31 or more leaves 0
+            const int sh = sk.shift, d = min(12, sh);
+            const uint32_t s1 = (uint32_t)min(sh, 31), s2 = (uint32_t)min(sh + 12, 31);
+            const uint32_t s3 = (uint32_t)min(sh - d, 31);
+            const uint32_t mask = (1u << d) - 1u, pre = (uint32_t)sk.prefix;
+            if (level > 1 && sk.prefix >= ((int64_t)1 << 31)) continue;      // no value can match
+            bool coarse = false;
+            for (int t = 16 * tid; t < t_end; t += 16 * kW32Threads) {
+                uint32_t p[16], q[16];
+                R.get16(t, p);
+                if ((W & 15) == 0) {
+                    R.get16(t + W, q);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) q[i] = R.get(t + W + i);
+                }
+                const int lim = t_end - t;                // starts t + i, i < lim
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int32_t S = (int32_t)(q[i] - p[i]);
+                    q[i] = S < 0 ? 0u - (uint32_t)S : (uint32_t)S;
+                }
+                if (level == 1) {
+                    uint32_t top = 0;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) top = max(top, q[i] >> s1);
+                    if (lim >= 16 && top < 4096u) {       // (nearly all)
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) atomicAdd(&h[q[i] >> s1], 1u);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const uint32_t k1 = q[i] >> s1;
+                            if (i < lim)
+                                atomicAdd(&h[k1 < 4096u ? k1 : 4096u + min(q[i] >> s2, 4095u)], 1u);
+                        }
+                        coarse = coarse || top >= 4096u;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        if (q[i] >> s1 == pre && i < lim)
+                            atomicAdd(&h[(q[i] >> s3) & mask], 1u);
+                }
+            }
+            coarse = __syncthreads_or(coarse);
+            // the counts to the global ones, and cleared for the next width
+            uint32_t* g = a.whist + ((int64_t)trial * a.nw + k) * kWsigBins;
+            const int nbins = level > 1 ? 1 << d : coarse ? kWsigBins : 4096;
+            for (int i = tid; i < nbins; i += kW32Threads) {
+                const uint32_t c = h[i];
+                if (c) {
+                    atomicAdd(&g[i], c);
+                    h[i] = 0;
+                }
+            }
+            __syncthreads();
         }
     }
 }
@@ -1782,8 +1917,19 @@ cudaError_t launch_width_sigma(const SearchArgs& a, cudaStream_t s, int64_t* nla
     if ((e = cudaFuncSetAttribute(wsig_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem)) != cudaSuccess)
         return e;
-    const dim3 hgrid((unsigned)ceil_div(a.nout, tile), a.ndm);
+    const dim3 hgrid((unsigned)std::min<int64_t>(ceil_div(a.nout, tile), kWsigBlocksPerTrial), a.ndm);
+    const int entries = kW32Tile + (a.wmax + 15) / 16 * 16 + 16;
+    const size_t smem32 = ((size_t)entries + kWsigBins) * sizeof(uint32_t);
+    if ((e = cudaFuncSetAttribute(wsig_hist32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem32)) != cudaSuccess)
+        return e;
+    const int64_t tiles32 = ceil_div(a.nout, kW32Tile);
     for (int level = 1; level <= kWsigPasses; ++level) {
+        ++*nlaunch;
+        // (the third digit and the fourth are rarely reached)
+        const int64_t gx = level <= 2 ? tiles32 : std::min<int64_t>(tiles32, kWsigBlocksPerTrial);
+        wsig_hist32_kernel<<<dim3((unsigned)gx, a.ndm), kW32Threads, smem32, s>>>(a, level, entries);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         ++*nlaunch;
         wsig_hist_kernel<<<hgrid, kWsigThreads, smem, s>>>(a, level, tile);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
