@@ -116,7 +116,9 @@ struct DedispJob {
     // left to the search.
     int32_t* lv;
     int64_t lv_pitch;
-    int64_t pattern;           // 1: tables of the pattern-row kernel
+    // 0: byte rows; 1: tables of the pattern-row kernel; k > 1: of that kernel, each tile
+    // summed by k blocks that add their parts to the output (zeros before)
+    int64_t pattern;
 };
 
 // Jobs of one dedispersion launch, passed by value as the kernel parameter.

@@ -251,10 +251,14 @@ __device__ __forceinline__ void add_rows(uint32_t (&acc)[kPatRD][kPatNJ], uint32
     }
 }
 
+// SPLIT: tiles of jobs with J.pattern > 1 are shared by that many blocks, each with a part
+// of the stages, whose sums are added to the zeroed output (plan.cpp, pattern_waves, has
+// when and the figures).
 // Warps 0-3 add pattern rows (six trials of the tile each), warps 4-14 form them
 // from the staged bytes, warp 15 issues the bulk copies.  The summing warps hold
 // six trials x 32 packed words per lane; their 32-bit sums are in tensor memory
 // (48 K words), where the 16-bit sums are added every 256 channels.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kPatThreads, 1)
 dedisp_patterns_kernel(const __grid_constant__ DedispBatch batch, int* status, uint64_t timeout_ns,
                        uint32_t one) {
@@ -274,14 +278,23 @@ dedisp_patterns_kernel(const __grid_constant__ DedispBatch batch, int* status, u
     // groups of eight time tiles, every DM tile of a group before the next group
     // (the windows of a group's rows stay in L2)
     constexpr int TG = 8;
-    const int64_t item = blk - batch.prefix[jb];
+    // (a tile of a split job belongs to J.pattern blocks, each with a part of its stages)
+    const int nparts = SPLIT ? (int)J.pattern : 1;
+    const int64_t item = (blk - batch.prefix[jb]) / nparts;
     const int64_t per = (int64_t)TG * J.ndt;
     const int64_t grp = item / per;
     const int64_t rem = item - grp * per;
     const int64_t gsz = min((int64_t)TG, (int64_t)J.ntt - grp * TG);
     const int dt = (int)(rem / gsz);
     const int tt = (int)(grp * TG + rem % gsz);
-    const TileDesc T = J.tiles[dt];
+    TileDesc T = J.tiles[dt];
+    if (SPLIT && nparts > 1) {
+        const int part = (int)((blk - batch.prefix[jb]) % nparts);
+        const int s0 = T.nstages * part / nparts, s1 = T.nstages * (part + 1) / nparts;
+        if (s0 == s1) return;                                  // the whole block
+        T.stage_begin += s0;
+        T.nstages = s1 - s0;
+    }
     const int64_t t0 = (int64_t)tt * kPatBT;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nst = T.nstages;
@@ -397,7 +410,7 @@ dedisp_patterns_kernel(const __grid_constant__ DedispBatch batch, int* status, u
             if (g) add_rows<1>(acc, rows, tab);
             __syncwarp();
             if (lane == 0) mbar_arrive(&row_free[rb]);
-            if (H.y) {   // add the 16-bit sums to the 32-bit sums
+            if (H.y || (SPLIT && s == nst - 1)) {   // add the 16-bit sums to the 32-bit sums
 #pragma unroll
                 for (int r = 0; r < kPatRD; ++r)
 #pragma unroll
@@ -437,7 +450,12 @@ dedisp_patterns_kernel(const __grid_constant__ DedispBatch batch, int* status, u
 #pragma unroll
                     for (int j = 0; j < kPatNJ; ++j) {
                         const int64_t t = t0 + e * kPatL + 32 * j + lane;
-                        if (t < J.nout) row[t] = (int32_t)v[j];
+                        if (t < J.nout) {
+                            if (!SPLIT || nparts == 1)
+                                row[t] = (int32_t)v[j];
+                            else                               // (zeroed before the launch)
+                                atomicAdd(&row[t], (int32_t)v[j]);
+                        }
                     }
                 }
             }
@@ -463,12 +481,14 @@ cudaError_t launch_dedisp_patterns(const DedispBatch& b, int* status, uint64_t t
                                    cudaStream_t s) {
     const int64_t total = b.prefix[b.njobs];
     if (total <= 0) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(dedisp_patterns_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+    // (the kernel without the parts of tiles is 1 to 2% faster)
+    bool split = false;
+    for (int j = 0; j < b.njobs; ++j) split = split || b.jobs[j].pattern > 1;
+    const auto k = split ? dedisp_patterns_kernel<true> : dedisp_patterns_kernel<false>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)kPatSmem);
     if (e != cudaSuccess) return e;
-    dedisp_patterns_kernel<<<(unsigned)total, kPatThreads, kPatSmem, s>>>(
-        b, status, timeout_ns, 1u);
+    k<<<(unsigned)total, kPatThreads, kPatSmem, s>>>(b, status, timeout_ns, 1u);
     return cudaGetLastError();
 }
 

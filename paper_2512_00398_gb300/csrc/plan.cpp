@@ -679,22 +679,67 @@ bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch) {
     return last_t0 + p->tiling.max_reach <= xt_pitch;
 }
 
+// Waves of `total` pattern-row blocks, in units of a whole tile's time, if the tiles of
+// the last *cols of the last input's ntt time columns (0: none) are shared by *parts
+// blocks each.  A block takes a tile's channels one after another for up to a
+// millisecond, and one block fits an SM: 320 blocks (375 trials, four gulps) on 152 SMs
+// took three such waves where 2.1 would do.  A part takes 1 / parts of a wave and
+// `fixed` more to fill its pipeline and to add its sums to the output; a
+// gain of less than 4% or 0.15 waves is left, as the kernel that takes parts of tiles is
+// 1 to 2% slower and tiles of high delays take longer than the others.  Measured, whole
+// tiles and parts by this rule, 4096 channels: 1500 trials x 9215 samples (2.07 waves)
+// 2.12 and 1.58 ms; 375 x 83968 (4.32) 4.06 and 3.64; 1500 x 129 000 (26.1) 12.80 and
+// 12.61; 750 x 8192 (0.84) 0.833, 0.869 split against the rule.
+double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total, int ntt, int* cols,
+                     int* parts) {
+    *cols = 0;
+    *parts = 1;
+    const int64_t sms = p->sm_count;
+    double best = (double)ceil_div(total, sms);
+    if (nq <= 0 || cycles <= 0) return best;
+    double limit = best - std::max(0.04 * best, 0.15);
+    const double fixed = 20000.0 * (double)nq / cycles;
+    const int max_parts = std::min(16, p->nchans / 64);
+    for (int c = 1; c <= std::min(ntt, 24) && c * nq <= 2 * sms; ++c)
+        for (int k = 2; k <= max_parts; ++k) {
+            const int64_t whole = total - c * nq, waves = ceil_div(whole, sms);
+            const double unit = 1.0 / k + fixed;
+            // parts that fit the idle SMs of the last whole wave, then waves of parts
+            const int64_t rest = c * nq * k - (waves * sms - whole) * (int64_t)(1.0 / unit);
+            const double t = (double)waves + (rest > 0 ? (double)ceil_div(rest, sms) * unit : 0.0);
+            if (t < limit) {
+                best = limit = t;
+                *cols = c;
+                *parts = k;
+            }
+        }
+    return best;
+}
+
 // Is a launch of njobs inputs of nout samples faster with pattern rows that take
 // `cycles` per time tile?  Both kernels keep one block per SM, so the one whose last
 // wave ends first, by the estimated cycles of its blocks: the pattern rows' larger
 // tiles (24 trials x 2048 samples against 15 x 2176) lose on short inputs, where a
 // wave is nearly empty, although they take fewer cycles per sum.  (The 1.03 leaves
-// near ties, within the estimates' error, to the byte rows.)
+// near ties, within the estimates' error, to the byte rows.)  Sharing tiles among
+// blocks (pattern_waves) makes up for that on many short inputs: 4096 channels, 375
+// trials, 4000 samples 0.833 ms by byte rows, 0.256 by parts of pattern rows; 2048
+// channels, 200 trials, 8192 samples 0.421 and 0.160.  There the tables must earn more
+// (1.25): they cost the plan's first call 2 to 5 ms.
 bool patterns_pay(const hp_plan* p, double cycles, int64_t nout, int njobs) {
     // the default tile shape of direct dedispersion, without fused remedian levels
     if (p->dedisp_cfg != kDefaultDedispConfig || p->sb_chans > 0 || p->fuse_levels) return false;
     if (cycles <= 0 || nout <= 0) return false;
     const DedispTiling& T = p->tiling;
     const int64_t nt = (int64_t)T.tiles.size(), nq = ceil_div(p->ndm(), kPatBD);
-    const double q = (double)ceil_div(ceil_div(nout, kPatBT) * nq * njobs, p->sm_count) * cycles / (double)nq;
+    const double tile = cycles / (double)nq;
+    const int64_t ntt = ceil_div(nout, kPatBT);
+    const double q = (double)ceil_div(ntt * nq * njobs, p->sm_count) * tile;
     const double t = (double)ceil_div(ceil_div(nout, T.BT) * nt * njobs, p->sm_count) *
                      byte_row_cycles((double)T.BD * p->nchans * T.BT);
-    return q * 1.03 < t;
+    int cols, parts;
+    return q * 1.03 < t ||
+           pattern_waves(p, cycles, nq, ntt * nq * njobs, (int)ntt, &cols, &parts) * tile * 1.25 < t;
 }
 
 bool use_patterns(const hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs) {
@@ -776,6 +821,34 @@ DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_
     J.lv_pitch = 0;
     J.pattern = pat ? 1 : 0;
     return J;
+}
+
+// Split the last time tiles of a launch of pattern-row jobs of plan p over several
+// blocks each (plan_internal.h).
+int split_tail(const hp_plan* p, DedispBatch* b, cudaStream_t s) {
+    if (b->njobs < 1 || b->njobs >= kMaxJobs) return HP_OK;
+    for (int j = 0; j < b->njobs; ++j)
+        if (b->jobs[j].pattern != 1) return HP_OK;
+    DedispJob& J = b->jobs[b->njobs - 1];
+    const int64_t nq = J.ndt;
+    int cols = 0, parts = 1;
+    pattern_waves(p, p->ptiling.cycles, nq, b->prefix[b->njobs], J.ntt, &cols, &parts);
+    if (cols == 0) return HP_OK;
+    DedispJob& Q = b->jobs[b->njobs];
+    Q = J;
+    const int64_t t1 = (int64_t)(J.ntt - cols) * kPatBT;
+    Q.xt += t1;
+    Q.out += t1;
+    Q.nout -= t1;
+    Q.ntt = cols;
+    Q.pattern = parts;
+    J.nout = t1;
+    J.ntt -= cols;
+    b->prefix[b->njobs] -= (int64_t)cols * nq;
+    b->prefix[b->njobs + 1] = b->prefix[b->njobs] + (int64_t)cols * nq * parts;
+    ++b->njobs;
+    return check_cuda(cudaMemset2DAsync(Q.out, (size_t)Q.out_pitch * 4, 0, (size_t)Q.nout * 4,
+                                        (size_t)p->ndm(), s));
 }
 
 // The dedispersion of the plan's own series also writes the second remedian
@@ -882,7 +955,8 @@ int run_dedisp(hp_plan* p, const uint8_t* fb, int64_t nsamps, const Layout& L, u
     B.prefix[0] = 0;
     B.prefix[1] = (int64_t)B.jobs[0].ntt * B.jobs[0].ndt;
     ti = stage_begin(p, HP_STAGE_DEDISP, s);
-    rc = check_cuda(launch_dedisp(p->dedisp_cfg, B, p->status, p->timeout_ns, s));
+    rc = split_tail(p, &B, s);
+    if (!rc) rc = check_cuda(launch_dedisp(p->dedisp_cfg, B, p->status, p->timeout_ns, s));
     stage_end(p, HP_STAGE_DEDISP, ti, s);
     if (!rc) ++p->launches;
     return rc;
@@ -1196,7 +1270,8 @@ int batch_enqueue(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
             db.jobs[0] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout);
             fuse_levels(db.jobs[0], L, ws);
             db.prefix[1] = (int64_t)db.jobs[0].ntt * db.jobs[0].ndt;
-            rc = check_cuda(launch_dedisp(b->cfg, db, p->status, p->timeout_ns, s));
+            rc = split_tail(p, &db, s);
+            if (!rc) rc = check_cuda(launch_dedisp(b->cfg, db, p->status, p->timeout_ns, s));
             if (rc) return rc;
             ++k;
         }

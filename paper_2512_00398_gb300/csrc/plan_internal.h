@@ -164,6 +164,10 @@ Layout make_layout(const hp_plan* p, int64_t nsamps, bool with_dedisp);
 int64_t xt_pitch_for(int64_t nsamps);
 int validate_search_input(const hp_plan* p, const void* ptr, int64_t nsamps);
 bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch);
+// Split the last time tiles of a launch of pattern-row jobs of plan p over several
+// blocks each where that fills a last wave that would be nearly empty (zeroes their
+// part of the output on s).
+int split_tail(const hp_plan* p, DedispBatch* b, cudaStream_t s);
 // One job of a launch of about `njobs` such jobs (the choice between the byte-row
 // and the pattern-row kernel depends on how many blocks the launch has).
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,

@@ -313,6 +313,7 @@ int enqueue_step(hp_stream* s, Step* st) {
                                             Ls[j].xt_pitch, work[j]->E - work[j]->B0, nullptr);
             rc = check_cuda(launch_rfi(r, m, &rfi_kernels));
         }
+        if (!rc && db.njobs > 0) rc = split_tail(p, &db, m);
         if (!rc && db.njobs > 0)
             rc = check_cuda(launch_dedisp(p->dedisp_cfg, db, p->status, p->timeout_ns, m));
         for (int j = 0; j < n && !rc && p->sb_chans > 0; ++j)
