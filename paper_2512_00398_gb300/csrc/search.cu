@@ -521,29 +521,76 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* warp
     return x - v + (warp > 0 ? warp_tot[warp - 1] : 0);
 }
 
-// Block-wide search of the bin holding rank k (0-based) in a histogram of
-// `bins` counts.  Returns the bin and the count of all earlier bins.
-__device__ void find_rank_bin(const uint32_t* hrow, int bins, int64_t k, int* bin_out,
-                              int64_t* before_out) {
-    __shared__ int64_t warp_tot[32];
+// Search by a block of kSelectThreads of the bin holding rank k (0-based) in a histogram
+// row of BINS counts: the bin, the count of all earlier bins, and the highest bin that
+// is not empty.  A warp reads its eighth of the row once, 512 bytes a load, and the one
+// whose part holds the rank finds it from its registers.  (1024 threads that walked
+// eight bins each, and again to find the bin, took 19.7 us for 750 rows, and a block
+// of 1024 leaves no more than two rows an SM.)
+constexpr int kSelectThreads = 256;
+template <int BINS>
+__device__ __forceinline__ void find_rank_bin(const uint32_t* hrow, int64_t k, int* bin_out,
+                                              int64_t* before_out, int* top_out) {
+    constexpr int kWarps = kSelectThreads / 32, kPart = BINS / kWarps, J = kPart / 128;
+    __shared__ int64_t warp_sum[kWarps];
+    __shared__ int warp_top[kWarps];
     __shared__ int s_bin;
     __shared__ int64_t s_before;
-    const int per = (bins + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * per, b1 = min(bins, b0 + per);
-    int64_t mine = 0;
-    for (int b = b0; b < b1; ++b) mine += hrow[b];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4 v[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+        v[j] = *reinterpret_cast<const uint4*>(hrow + warp * kPart + 128 * j + 4 * lane);
+    int64_t sum = 0;
+    int top = -1;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        sum += (int64_t)v[j].x + v[j].y + v[j].z + v[j].w;
+        const int i = warp * kPart + 128 * j + 4 * lane;
+        if (v[j].x | v[j].y | v[j].z | v[j].w)
+            top = i + (v[j].w ? 3 : v[j].z ? 2 : v[j].y ? 1 : 0);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    }
+    if (lane == 0) {
+        warp_sum[warp] = sum;
+        warp_top[warp] = top;
+    }
     if (threadIdx.x == 0) { s_bin = -1; s_before = 0; }
-    const int64_t excl = block_exclusive_scan(mine, warp_tot);   // (synchronises)
-    if (excl <= k && k < excl + mine) {
-        int64_t c = excl;
-        for (int b = b0; b < b1; ++b) {
-            if (k < c + hrow[b]) { s_bin = b; s_before = c; break; }
-            c += hrow[b];
+    __syncthreads();
+    int64_t c = 0;
+    for (int w = 0; w < kWarps; ++w) {
+        c += w < warp ? warp_sum[w] : 0;
+        top = max(top, warp_top[w]);
+    }
+    if (c <= k && k < c + sum) {
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t q[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+            const int64_t mine = (int64_t)q[0] + q[1] + q[2] + q[3];
+            int64_t x = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t u = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += u;
+            }
+            int64_t e = c + x - mine;                      // counts before this lane's four
+            if (e <= k && k < e + mine) {
+                int i = 0;
+                for (; k >= e + q[i]; ++i) e += q[i];
+                s_bin = warp * kPart + 128 * j + 4 * lane + i;
+                s_before = e;
+            }
+            c += __shfl_sync(0xffffffffu, x, 31);
         }
     }
     __syncthreads();
     *bin_out = s_bin;
     *before_out = s_before;
+    *top_out = top;
 }
 
 // sigma = 1.4826.. x MAD and the integer thresholds ceil(thr * sigma * sqrt(W)) of a
@@ -565,33 +612,21 @@ __device__ __forceinline__ void write_thresholds(const SearchArgs& a, int trial,
     }
 }
 
-__global__ void __launch_bounds__(1024) mad_select_kernel(const __grid_constant__ SearchArgs a) {
+__global__ void __launch_bounds__(kSelectThreads) mad_select_kernel(const __grid_constant__ SearchArgs a) {
     pdl_wait();
     const int trial = blockIdx.x;
     uint32_t* hrow = a.hist + (int64_t)trial * kHistBins;
     const int64_t k = (a.nout - 1) / 2;
-    if (a.ybound) {
-        // an upper bound of max |y| from the highest non-empty bin: exact below
-        // kHistFine, the top of a coarse bin above, none for the last coarse bin
-        __shared__ int s_top;
-        if (threadIdx.x == 0) s_top = -1;
-        __syncthreads();
-        int top = -1;
-        for (int b = threadIdx.x; b < kHistBins; b += blockDim.x)
-            if (hrow[b]) top = b;
-        if (top >= 0) atomicMax(&s_top, top);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const int t = s_top;
-            a.ybound[trial] = t < 0 ? 0
-                          : t < kHistFine ? (int64_t)t
-                          : t == kHistBins - 1 ? -1
-                          : ((int64_t)(t - kHistFine + 1) << 12) - 1;
-        }
-    }
-    int bin;
+    int bin, top;
     int64_t before;
-    find_rank_bin(hrow, kHistBins, k, &bin, &before);
+    find_rank_bin<kHistBins>(hrow, k, &bin, &before, &top);
+    // an upper bound of max |y| from the highest non-empty bin: exact below
+    // kHistFine, the top of a coarse bin above, none for the last coarse bin
+    if (a.ybound && threadIdx.x == 0)
+        a.ybound[trial] = top < 0 ? 0
+                        : top < kHistFine ? (int64_t)top
+                        : top == kHistBins - 1 ? -1
+                        : ((int64_t)(top - kHistFine + 1) << 12) - 1;
     if (threadIdx.x == 0) {
         a.refine_bucket[trial] = bin < kHistFine ? -1 : bin - kHistFine;
         a.refine_rank[trial] = k - before;
@@ -632,14 +667,15 @@ __global__ void __launch_bounds__(256) mad_refine_hist_kernel(const __grid_const
         if (h[i]) atomicAdd(&g[i], h[i]);
 }
 
-__global__ void __launch_bounds__(1024) mad_refine_select_kernel(const __grid_constant__ SearchArgs a) {
+__global__ void __launch_bounds__(kSelectThreads) mad_refine_select_kernel(const __grid_constant__ SearchArgs a) {
     pdl_wait();
     const int trial = blockIdx.x;
     const int32_t B = a.refine_bucket[trial];
     if (B < 0) return;
-    int bin;
+    int bin, top;
     int64_t before;
-    find_rank_bin(a.hist + (int64_t)trial * kHistBins, kHistFine, a.refine_rank[trial], &bin, &before);
+    find_rank_bin<kHistFine>(a.hist + (int64_t)trial * kHistBins, a.refine_rank[trial], &bin, &before,
+                             &top);
     write_thresholds(a, trial, ((int64_t)B << 12) + bin);
 }
 
@@ -1857,16 +1893,18 @@ __global__ void __launch_bounds__(kW32Threads, 2) wsig_hist32_kernel(const __gri
     }
 }
 
-__global__ void __launch_bounds__(1024) wsig_select_kernel(const __grid_constant__ SearchArgs a,
+__global__ void __launch_bounds__(kSelectThreads) wsig_select_kernel(const __grid_constant__ SearchArgs a,
                                                            int level) {
     const int64_t idx = blockIdx.x;                       // trial * nw + k
     WsigState st = a.wstate[idx];
     if (st.level != level) return;                        // the whole block
     uint32_t* hrow = a.whist + idx * kWsigBins;
-    const int nbins = level == 1 ? kWsigBins : 1 << min(12, st.shift);
-    int bin;
+    int bin, top;
     int64_t before;
-    find_rank_bin(hrow, nbins, st.rank, &bin, &before);
+    if (level == 1)
+        find_rank_bin<kWsigBins>(hrow, st.rank, &bin, &before, &top);
+    else                                                  // (zeros past the digit's bins)
+        find_rank_bin<4096>(hrow, st.rank, &bin, &before, &top);
     if (threadIdx.x == 0) {
         if (level == 1 && bin == kWsigBins - 1) {
             // beyond what the first pass resolves: every digit from the top
@@ -1934,7 +1972,7 @@ cudaError_t launch_width_sigma(const SearchArgs& a, cudaStream_t s, int64_t* nla
         wsig_hist_kernel<<<hgrid, kWsigThreads, smem, s>>>(a, level, tile);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         ++*nlaunch;
-        wsig_select_kernel<<<(unsigned)pairs, 1024, 0, s>>>(a, level);
+        wsig_select_kernel<<<(unsigned)pairs, kSelectThreads, 0, s>>>(a, level);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     ++*nlaunch;
@@ -2040,11 +2078,11 @@ cudaError_t launch_walkers(const SearchArgs& a, const BaselineCtx& bc, cudaStrea
         hist(std::integral_constant<int, 32>{});
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     ++*nlaunch;
-    if ((e = launch_pdl(mad_select_kernel, dim3(ndm), 1024, 0, s, a)) != cudaSuccess) return e;
+    if ((e = launch_pdl(mad_select_kernel, dim3(ndm), kSelectThreads, 0, s, a)) != cudaSuccess) return e;
     ++*nlaunch;
     if ((e = launch_pdl(mad_refine_hist_kernel, hgrid, 256, 0, s, a, yvec)) != cudaSuccess) return e;
     ++*nlaunch;
-    if ((e = launch_pdl(mad_refine_select_kernel, dim3(ndm), 1024, 0, s, a)) != cudaSuccess) return e;
+    if ((e = launch_pdl(mad_refine_select_kernel, dim3(ndm), kSelectThreads, 0, s, a)) != cudaSuccess) return e;
     if (a.stats_only) return cudaSuccess;
     if (a.width_sigma && (e = launch_width_sigma(a, s, nlaunch)) != cudaSuccess) return e;
     if (a.ndec > 0) {
