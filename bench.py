@@ -41,6 +41,11 @@ METRIC = "DM-trial·samples/s"
 # configuration reports null until it is captured again.
 DEDISP_TRAFFIC = {"source_sha256_16": "0e82e2697ab3fb83", "bytes": (6.095e9 + 1.010e9) * 955060 / 168628,
                   "ndm": 1500, "nchans": 4096, "nsamps": 1 << 20, "config": 17}
+# The same of the pattern-row kernel, which the default configuration runs on this
+# workload (profiles/dedisp_patterns_kernel_fast_4096ch.md).
+PATTERN_TRAFFIC = {"source_sha256_16": "759dd0ca1211772d",
+                   "bytes": (9.713e9 + 1.007e9) * 955060 / 168628,
+                   "ndm": 1500, "nchans": 4096, "nsamps": 1 << 20, "config": 17}
 # The same for the two stages of the sub-band variant (64-channel sub-bands, groups
 # of 8 trials): DRAM bytes of one step, captured on the 2^18-sample case
 # (profiles/subband_fast_4096ch.md).  Stage 1's traffic grows with its byte-adds
@@ -236,9 +241,9 @@ def subband_traffic(w, config, S, G):
 PRMT_PER_WORD = 2.0
 
 
-def dedisp_traffic(w, config):
-    sha = source_sha("dedisp.cu")
-    t = DEDISP_TRAFFIC
+def dedisp_traffic(w, config, patterns):
+    sha = source_sha("patterns.cu" if patterns else "dedisp.cu")
+    t = PATTERN_TRAFFIC if patterns else DEDISP_TRAFFIC
     if (sha != t["source_sha256_16"] or w.ndm != t["ndm"] or w.obs.nchans != t["nchans"]
             or w.obs.nsamps != t["nsamps"] or config != t["config"]):
         return None
@@ -454,11 +459,15 @@ def run_ours(args):
         peak_adds = 2.0 * peaks["int_add_ops_per_s"]
         achieved = adds / (dd_ms * 1e-3)
         cfg = int(plan.get_param("dedisp_config"))
-        traffic = dedisp_traffic(w, cfg)
+        # the default tile shape's plans take pattern rows (sums of up to four channels
+        # shared between trials): fewer additions than the byte-adds counted here
+        patterns = cfg == 17 and int(plan.get_param("fuse_levels")) == 0
+        traffic = dedisp_traffic(w, cfg, patterns)
         alg_bytes = float(o.nchans) * o.nsamps + 4.0 * w.ndm * nout
         hbm_peak = measured_hbm_gbs()
         line["roofline"] = {
-            "bound": "alu", "kernel": "dedisp_rows_kernel", "achieved": achieved / 1e12,
+            "bound": "alu", "kernel": "dedisp_patterns_kernel" if patterns else "dedisp_rows_kernel",
+            "achieved": achieved / 1e12,
             "peak": peak_adds / 1e12, "unit": "Tadd/s", "frac": achieved / peak_adds,
             "traffic": traffic,
             "algorithmic": f"{w.ndm} trials x {o.nchans} ch x {nout} samples = {adds:.3e} "
@@ -469,8 +478,9 @@ def run_ours(args):
                     "peak_gbs": hbm_peak, "basis": "MEASURED_PEAKS.json hbm_gbs (of measured)"},
             # each 4-sample word costs prmt_per_word ALU-pipe PRMTs (align, then
             # one or two splits); the measured PRMT rate is the ALU pipe's rate
-            "frac_vs_alu_design_ceiling": achieved / (peaks["prmt_ops_per_s"] * 4.0
-                                                      / PRMT_PER_WORD),
+            # (of the byte rows)
+            "frac_vs_alu_design_ceiling": None if patterns else
+                achieved / (peaks["prmt_ops_per_s"] * 4.0 / PRMT_PER_WORD),
             "config": cfg,
             "peak_basis": "measured int32 add issue rate x 2 (16-bit SWAR lanes); "
                           f"int32 {peaks['int_add_ops_per_s'] / 1e12:.2f} Tops/s, PRMT "
@@ -482,7 +492,7 @@ def run_ours(args):
         # shared-memory loads: NW + 1 row words per lane, channel and trial for NW
         # words of 4 samples (byte-row kernels), against the measured LDS.32 rate
         shape = hp.hp_dedisp_config(cfg)
-        if True:
+        if not patterns:
             lds_bytes = adds * (shape["NW"] + 1) / shape["NW"]
             line["roofline"]["lds"] = {
                 "achieved_tbs": lds_bytes / (dd_ms * 1e-3) / 1e12,
@@ -793,7 +803,7 @@ def config_line(w, ms, stages, cands, s, peaks, hbm_peak, nout):
     return {
         "value": w.ndm * nout / (ms * 1e-3), "unit": METRIC, "ms_per_step": ms,
         "rtf": o.duration / (ms * 1e-3), "stages_ms": stages,
-        "roofline": {"bound": "alu", "kernel": "dedisp_rows_kernel",
+        "roofline": {"bound": "alu", "kernel": "dedisp_patterns_kernel or dedisp_rows_kernel, by size",
                      "achieved": adds / (stages["dedisp"] * 1e-3) / 1e12,
                      "peak": peak_adds / 1e12, "unit": "Tadd/s",
                      "frac": adds / (stages["dedisp"] * 1e-3) / peak_adds},
