@@ -14,9 +14,10 @@
 // Device memory (one allocation): per step slot j < max_batch a search
 // workspace for G + H samples and a candidate buffer; per beam slot a ring of
 // R = ceil(H / G) + 1 gulps ([G][nchans] each; the buffer of gulp g is gulps
-// g - R + 1 .. g) and two [ndm][nw] carry arrays used alternately.  Host
-// uploads, kernels and result copies of a step are ordered on one stream, so a
-// ring slot is rewritten only after every step that read it has finished.
+// g - R + 1 .. g) and two [ndm][nw] carry arrays used alternately.  Kernels and
+// result copies of the steps are ordered on one stream; a step's uploads run on
+// another, beside the step before, once that one's transpose -- the only reader
+// of the rings -- is done, so a ring slot is rewritten only after every read of it.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -112,6 +113,10 @@ struct hp_stream {
     cudaStream_t main = nullptr;
     std::vector<cudaStream_t> side;
     cudaEvent_t fork = nullptr;
+    // host-to-device copies of the gulps; `copied` after a step's, `ring_free` on main
+    // after a step's transpose, the last reader of the rings
+    cudaStream_t copy = nullptr;
+    cudaEvent_t copied = nullptr, ring_free = nullptr;
     std::vector<cudaEvent_t> joins;
     std::thread th;
     std::mutex mu;
@@ -264,12 +269,20 @@ int enqueue_step(hp_stream* s, Step* st) {
     cudaStream_t m = s->main;
     const size_t gbytes = (size_t)s->G * s->nch;
     int rc = HP_OK;
-    // this step's gulps into their ring slots (after every earlier step on m)
+    // this step's gulps into their ring slots, on a stream of their own: a slot may hold
+    // the oldest gulp that the step before reads, so after that step's transpose, but
+    // beside its dedispersion and searches (four gulps of 32 MB: 0.5 of a step's 3.5 ms
+    // when the copies stood on m)
+    rc = check_cuda(cudaStreamWaitEvent(s->copy, s->ring_free, 0));
+    if (rc) return rc;
     for (const Item& it : st->items) {
         uint8_t* dst = s->slots[it.slot].ring + (size_t)(it.index % s->R) * gbytes;
-        rc = check_cuda(cudaMemcpyAsync(dst, it.host, gbytes, cudaMemcpyHostToDevice, m));
+        rc = check_cuda(cudaMemcpyAsync(dst, it.host, gbytes, cudaMemcpyHostToDevice, s->copy));
         if (rc) return rc;
     }
+    rc = check_cuda(cudaEventRecord(s->copied, s->copy));
+    if (!rc) rc = check_cuda(cudaStreamWaitEvent(m, s->copied, 0));
+    if (rc) return rc;
     TransposeBatch tb;
     std::memset(&tb, 0, sizeof(tb));
     DedispBatch db;
@@ -307,6 +320,7 @@ int enqueue_step(hp_stream* s, Step* st) {
         tb.njobs = n;
         db.njobs = p->sb_chans > 0 ? 0 : n;
         rc = check_cuda(launch_transpose_batch(tb, m));
+        if (!rc) rc = check_cuda(cudaEventRecord(s->ring_free, m));
         int64_t rfi_kernels = 0;
         for (int j = 0; j < n && !rc && p->rfi; ++j) {   // RFI mitigation per searched buffer
             const RfiArgs r = make_rfi_args(p, Ls[j], s->ws[j], nullptr, s->ws[j] + Ls[j].xt,
@@ -384,6 +398,7 @@ void scheduler(hp_stream* s) {
                 // nothing more is enqueued after a failed call: wait for the
                 // device, then report the step's gulps with the error
                 lk.unlock();
+                cudaStreamSynchronize(s->copy);
                 cudaStreamSynchronize(s->main);
                 for (cudaStream_t x : s->side) cudaStreamSynchronize(x);
                 lk.lock();
@@ -431,11 +446,15 @@ int copy_plan(const hp_plan* t, int64_t raw_capacity, hp_plan** out) {
 }
 
 void release(hp_stream* s) {
+    if (s->copy) cudaStreamSynchronize(s->copy);
     if (s->main) cudaStreamSynchronize(s->main);
     for (cudaStream_t x : s->side) {
         cudaStreamSynchronize(x);
         cudaStreamDestroy(x);
     }
+    if (s->copied) cudaEventDestroy(s->copied);
+    if (s->ring_free) cudaEventDestroy(s->ring_free);
+    if (s->copy) cudaStreamDestroy(s->copy);
     for (cudaEvent_t e : s->joins) cudaEventDestroy(e);
     if (s->fork) cudaEventDestroy(s->fork);
     if (s->main) cudaStreamDestroy(s->main);
@@ -530,7 +549,9 @@ int hp_stream_open(hp_stream** out, const hp_plan* tmpl, const hp_stream_config*
     s->pinned = (uint8_t*)hbuf;
     std::memset(s->pinned, 0, kSets * s->set_bytes);
     rc = check_cuda(cudaStreamCreateWithFlags(&s->main, cudaStreamNonBlocking));
-    if (!rc) rc = check_cuda(cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming));
+    if (!rc) rc = check_cuda(cudaStreamCreateWithFlags(&s->copy, cudaStreamNonBlocking));
+    for (cudaEvent_t* e : {&s->fork, &s->copied, &s->ring_free})
+        if (!rc) rc = check_cuda(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     for (int j = 0; j < mb && !rc; ++j) {
         cudaStream_t x;
         cudaEvent_t e;
