@@ -1017,7 +1017,7 @@ __global__ void __launch_bounds__(kDetectThreads) detect_kernel(const __grid_con
 // counting each candidate up on the list by itself, took 87 of the 110 ms that the
 // search of 4096 channels x 2^20 samples x 1500 trials with masked interference needs
 // there, this 38 (and 14 -> 0.8 ms in tail_kernel); a single list of 4e5 candidates
-// 0.94 -> 0.71 ms.  A quiet series pays 2.32 -> 2.4 ms for the registers (of 173).
+// 0.94 -> 0.71 ms.  A quiet series pays 2.32 -> 2.50 ms for the registers (of 173).
 constexpr int kDWThreads = 128;
 constexpr int kDWPer = 16;                          // consecutive starts per thread
 constexpr int kDWChunk = kDWThreads * kDWPer;       // starts per chunk
