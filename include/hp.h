@@ -401,7 +401,8 @@ int hp_merge_static(const hp_raw_cand* raw_dev, const int64_t* nraw_dev, int64_t
 /* Device memory of the plan (its tables and, unless a workspace is bound, its
  * search workspace) from a caller's allocator instead of cudaMalloc/cudaFree,
  * e.g. a framework's caching allocator.  alloc returns a device pointer
- * aligned to 256 bytes or NULL; free gets back the pointer and its size.  The
+ * aligned to 256 bytes or NULL, ready for use on the stream of the call that asked
+ * for it; free gets back the pointer and its size.  The
  * plan synchronises the device before it frees anything, so the memory is idle
  * when free is called.  Both NULL restores cudaMalloc.  Memory obtained from
  * the previous allocator is returned to it first.  Not thread-safe with

@@ -575,7 +575,30 @@ Layout make_layout(const hp_plan* p, int64_t nsamps, bool with_dedisp) {
     return L;
 }
 
-int ensure_device_tables(hp_plan* p) {
+// Constant tables from (pageable) host vectors, on the device when finish() returns:
+// any stream may launch the kernel that reads them.  The copies run on the call's own
+// stream, after whatever still uses memory that a stream-ordered allocator hands out
+// again.  (cudaMemcpy alone may return while its last piece is still on the way, on a
+// stream that non-blocking ones do not wait for.)
+struct TableUpload {
+    cudaStream_t s;
+    int rc = HP_OK;
+    explicit TableUpload(cudaStream_t stream) : s(stream) {
+        // under capture the legacy stream, as nothing may wait for s
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        rc = check_cuda(cudaStreamIsCapturing(s, &cap));
+        if (cap != cudaStreamCaptureStatusNone) s = cudaStreamLegacy;
+    }
+    void put(void* dst, const void* src, size_t bytes) {
+        if (!rc && bytes) rc = check_cuda(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+    }
+    int finish() {
+        const int e = check_cuda(cudaStreamSynchronize(s));
+        return rc ? rc : e;
+    }
+};
+
+int ensure_device_tables(hp_plan* p, cudaStream_t s) {
     const int64_t sb_key = p->sb_chans > 0 ? ((int64_t)p->sb_chans << 32) | p->sb_group : 0;
     if (p->tables && p->tables_cfg == p->dedisp_cfg && p->tables_sb == sb_key) return HP_OK;
     int dev = 0;
@@ -622,16 +645,15 @@ int ensure_device_tables(hp_plan* p) {
     int rc = plan_alloc(p, total, &mem);
     if (rc) return rc;
     uint8_t* b = (uint8_t*)mem;
-    auto put = [&](size_t at, const void* src, size_t bytes) {
-        if (!rc && bytes) rc = check_cuda(cudaMemcpy(b + at, src, bytes, cudaMemcpyHostToDevice));
-    };
-    put(o_status, &prev_status, sizeof(int));
-    put(o_tiles, T.tiles.data(), T.tiles.size() * sizeof(TileDesc));
-    put(o_stages, T.stages.data(), T.stages.size() * sizeof(StageDesc));
-    put(o_chans, T.chans.data(), T.chans.size() * sizeof(ChanDesc));
-    put(o_addr, T.addr.data(), T.addr.size() * sizeof(uint32_t));
-    put(o_widths, p->widths.data(), p->widths.size() * sizeof(int32_t));
-    put(o_sbtop, sbtop.data(), sbtop.size() * sizeof(int32_t));
+    TableUpload up(s);
+    up.put(b + o_status, &prev_status, sizeof(int));
+    up.put(b + o_tiles, T.tiles.data(), T.tiles.size() * sizeof(TileDesc));
+    up.put(b + o_stages, T.stages.data(), T.stages.size() * sizeof(StageDesc));
+    up.put(b + o_chans, T.chans.data(), T.chans.size() * sizeof(ChanDesc));
+    up.put(b + o_addr, T.addr.data(), T.addr.size() * sizeof(uint32_t));
+    up.put(b + o_widths, p->widths.data(), p->widths.size() * sizeof(int32_t));
+    up.put(b + o_sbtop, sbtop.data(), sbtop.size() * sizeof(int32_t));
+    rc = up.finish();
     if (rc) {
         plan_free(p, mem, total);
         return rc;
@@ -776,13 +798,12 @@ int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cuda
     int rc = plan_alloc(p, off, &mem);
     if (rc) return HP_OK;   // no room: the byte rows run
     uint8_t* b = (uint8_t*)mem;
-    auto put = [&](size_t at, const void* src, size_t bytes) {
-        if (!rc) rc = check_cuda(cudaMemcpy(b + at, src, bytes, cudaMemcpyHostToDevice));
-    };
-    put(o_tiles, Q.tiles.data(), Q.tiles.size() * sizeof(TileDesc));
-    put(o_stages, Q.stages.data(), Q.stages.size() * sizeof(StageDesc));
-    put(o_chans, Q.chans.data(), Q.chans.size() * sizeof(ChanDesc));
-    put(o_addr, Q.addr.data(), Q.addr.size() * sizeof(uint32_t));
+    TableUpload up(s);
+    up.put(b + o_tiles, Q.tiles.data(), Q.tiles.size() * sizeof(TileDesc));
+    up.put(b + o_stages, Q.stages.data(), Q.stages.size() * sizeof(StageDesc));
+    up.put(b + o_chans, Q.chans.data(), Q.chans.size() * sizeof(ChanDesc));
+    up.put(b + o_addr, Q.addr.data(), Q.addr.size() * sizeof(uint32_t));
+    rc = up.finish();
     if (rc) {
         plan_free(p, mem, off);
         return rc;
@@ -1141,7 +1162,7 @@ bool autotune_candidate(int c) { return c >= 0 && c < kNumDedispConfigs; }
 // time one transpose + dedispersion of `p` on `s` with events (synchronising)
 int time_dedisp(hp_plan* p, const uint8_t* fb, int64_t nsamps, cudaStream_t s, int reps,
                 float* ms_out) {
-    int rc = ensure_device_tables(p);
+    int rc = ensure_device_tables(p, s);
     if (rc) return rc;
     Layout L = make_layout(p, nsamps, true);
     uint8_t* ws = nullptr;
@@ -1203,7 +1224,7 @@ int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
         int rc = validate_search_input(p, fbs ? fbs[i] : nullptr, nsamps[i]);
         if (rc) return rc;
         if (p->sb_chans <= 0) p->dedisp_cfg = b->cfg;   // sub-band files keep their stage-1 shape
-        rc = ensure_device_tables(p);
+        rc = ensure_device_tables(p, s);
         if (rc) return rc;
         (*layouts)[i] = make_layout(p, nsamps[i], true);
         rc = prepare_patterns(p, (*layouts)[i].nout, (*layouts)[i].xt_pitch, 1, s);
@@ -1579,7 +1600,7 @@ int hp_rfi_clean(hp_plan* p, const uint8_t* fb, int64_t nsamps, void* stream, ui
                  uint8_t* chan_flag, uint8_t* samp_flag, int32_t* chan_median) {
     if (!p || !fb || nsamps < 1 || nsamps >= kMaxSamples) return HP_ERR_INVALID_ARG;
     if (cleaned == fb) return HP_ERR_INVALID_ARG;
-    int rc = ensure_device_tables(p);
+    int rc = ensure_device_tables(p, (cudaStream_t)stream);
     if (rc) return rc;
     Layout L = make_layout(p, std::max<int64_t>(nsamps, (int64_t)p->maxd + 1), true);
     uint8_t* ws = nullptr;
@@ -1610,7 +1631,7 @@ int hp_dedisperse(hp_plan* p, const uint8_t* fb, int64_t nsamps, int32_t* out, i
     if (rc) return rc;
     const int64_t nout = nsamps - p->maxd;
     if (!out || pitch < nout || (pitch & 3) || ((uintptr_t)out & 15u)) return HP_ERR_INVALID_ARG;
-    rc = ensure_device_tables(p);
+    rc = ensure_device_tables(p, (cudaStream_t)stream);
     if (rc) return rc;
     Layout L = make_layout(p, nsamps, true);
     uint8_t* ws = nullptr;
@@ -1624,7 +1645,7 @@ int hp_detect(hp_plan* p, const int32_t* series, int64_t nout, int64_t pitch, vo
     if (!p || !series || !raw_out || !raw_out->data || !raw_out->count || raw_out->capacity < 0)
         return HP_ERR_INVALID_ARG;
     if (nout <= p->wmax || pitch < nout) return HP_ERR_NSAMPS_TOO_SHORT;
-    int rc = ensure_device_tables(p);
+    int rc = ensure_device_tables(p, (cudaStream_t)stream);
     if (rc) return rc;
     Layout L = make_layout(p, nout + p->maxd, false);
     uint8_t* ws = nullptr;
@@ -1651,7 +1672,7 @@ int hp_merge(hp_plan* p, const hp_raw_cand* raw, const int64_t* nraw, int64_t ra
     if (!p || !raw || !nraw || !sigma || !out || !out->data || !out->count || out->capacity < 0 ||
         raw_capacity < 0)
         return HP_ERR_INVALID_ARG;
-    int rc = ensure_device_tables(p);
+    int rc = ensure_device_tables(p, (cudaStream_t)stream);
     if (rc) return rc;
     // the merge scratch is sized by the plan's raw capacity
     if (raw_capacity > p->raw_capacity) return HP_ERR_INVALID_ARG;
@@ -1671,7 +1692,7 @@ int hp_search(hp_plan* p, const uint8_t* fb, int64_t nsamps, void* stream, hp_ca
     int rc = validate_search_input(p, fb, nsamps);
     if (rc) return rc;
     if (!out || !out->data || !out->count || out->capacity < 0) return HP_ERR_INVALID_ARG;
-    rc = ensure_device_tables(p);
+    rc = ensure_device_tables(p, (cudaStream_t)stream);
     if (rc) return rc;
     Layout L = make_layout(p, nsamps, true);
     uint8_t* ws = nullptr;
@@ -1752,7 +1773,7 @@ int hp_plan_autotune(hp_plan* p, const uint8_t* fb, int64_t nsamps, void* stream
     }
     p->dedisp_cfg = best >= 0 ? best : keep;
     if (best >= 0) p->dedisp_cfg_set = true;
-    rc = ensure_device_tables(p);
+    rc = ensure_device_tables(p, s);
     if (rc) return rc;
     if (best_config) *best_config = p->dedisp_cfg;
     if (best_ms) *best_ms = best_t;
@@ -1916,7 +1937,7 @@ int hp_batch_autotune(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsa
     if (rc) return rc;
     for (hp_plan* p : b->plans) {
         if (p->sb_chans <= 0) p->dedisp_cfg = b->cfg;
-        rc = ensure_device_tables(p);
+        rc = ensure_device_tables(p, s);
         if (rc) return rc;
     }
     if (best_config) *best_config = b->cfg;

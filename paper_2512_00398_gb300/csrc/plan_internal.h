@@ -142,7 +142,9 @@ namespace hp {
 int check_cuda(cudaError_t e);
 int plan_alloc(hp_plan* p, size_t bytes, void** out);
 void plan_free(hp_plan* p, void* ptr, size_t bytes);
-int ensure_device_tables(hp_plan* p);
+// Build and upload the constant tables if they are missing or of another tile shape; s: the
+// stream of the call (waited for).
+int ensure_device_tables(hp_plan* p, cudaStream_t s);
 int ensure_workspace(hp_plan* p, size_t need, uint8_t** base);
 // Tables of the pattern-row kernel for the plan's direct delays; false (T left
 // empty) where they cannot be laid out.

@@ -494,7 +494,7 @@ int hp_stream_open(hp_stream** out, const hp_plan* tmpl, const hp_stream_config*
     s->nw = p->nw();
     if (s->R > kMaxRing) { release(s); return HP_ERR_INVALID_ARG; }
     if (cudaGetDevice(&s->device) != cudaSuccess) { release(s); return HP_ERR_CUDA; }
-    rc = ensure_device_tables(p);
+    rc = ensure_device_tables(p, nullptr);
     if (rc) { release(s); return rc; }
 
     // sizes: step slots (search workspace + candidates), beam slots (ring + carries)
