@@ -32,8 +32,11 @@ namespace hp {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// The status of a runtime call.  A failure is reported here once: the thread's last
+// error is cleared, or the next launch's cudaGetLastError would report it again.
 int check_cuda(cudaError_t e) {
     if (e == cudaSuccess) return HP_OK;
+    (void)cudaGetLastError();
     if (e == cudaErrorMemoryAllocation) return HP_ERR_OOM;
     return HP_ERR_CUDA;
 }
@@ -777,7 +780,7 @@ int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cuda
     if (p->pat_estimate == 0) p->pat_estimate = estimate_patterns(p);
     if (!patterns_pay(p, p->pat_estimate, nout, njobs)) return HP_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    if (check_cuda(cudaStreamIsCapturing(s, &cap)) || cap != cudaStreamCaptureStatusNone)
         return HP_OK;
     DedispTiling& Q = p->ptiling;
     if (!Q.pattern && !build_patterns(p, &Q)) {
@@ -796,7 +799,11 @@ int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cuda
     const size_t o_addr = take(Q.addr.size() * sizeof(uint32_t));
     void* mem = nullptr;
     int rc = plan_alloc(p, off, &mem);
-    if (rc) return HP_OK;   // no room: the byte rows run
+    if (rc) {               // no room: the byte rows run, from now on (no call asks again)
+        Q = DedispTiling();
+        p->pat_estimate = -1;
+        return HP_OK;
+    }
     uint8_t* b = (uint8_t*)mem;
     TableUpload up(s);
     up.put(b + o_tiles, Q.tiles.data(), Q.tiles.size() * sizeof(TileDesc));
@@ -1582,6 +1589,7 @@ int hp_plan_set_allocator(hp_plan* p, hp_alloc_fn alloc, hp_free_fn free_fn, voi
         p->ws_own_bytes = 0;
         if (st != 0) p->pending_status = st;
     }
+    if (!p->ptables) p->pat_estimate = 0;   // the new allocator may have room for the tables
     p->alloc_fn = alloc;
     p->free_fn = free_fn;
     p->alloc_ctx = ctx;

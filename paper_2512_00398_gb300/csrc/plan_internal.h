@@ -86,7 +86,7 @@ struct hp_plan {
     // input that the pattern-row kernel is estimated to be faster on.
     hp::DedispTiling ptiling;
     double pat_estimate = 0;           // SM cycles per time tile, all DM tiles, from a few of them
-                                       // (0: not estimated yet, < 0: no tables can be laid out)
+                                       // (0: not estimated yet, < 0: no tables can be laid out or held)
     void* ptables = nullptr;
     size_t ptables_bytes = 0;
     int sm_count = 148;
