@@ -773,6 +773,15 @@ bool use_patterns(const hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs) {
            patterns_pay(p, Q.cycles, nout, njobs);
 }
 
+// While it lives, this thread's allocations and copies are allowed beside another
+// stream's capture, which would otherwise (in the global mode, torch's default) be
+// invalidated by them.
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCaptures() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s) {
     if (p->ptables || p->pat_estimate < 0 || p->dedisp_cfg != kDefaultDedispConfig ||
         p->sb_chans > 0 || p->fuse_levels)
@@ -797,6 +806,7 @@ int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cuda
     const size_t o_stages = take(Q.stages.size() * sizeof(StageDesc));
     const size_t o_chans = take(Q.chans.size() * sizeof(ChanDesc));
     const size_t o_addr = take(Q.addr.size() * sizeof(uint32_t));
+    const BesideCaptures beside;   // (a later call than the plan's first may come here)
     void* mem = nullptr;
     int rc = plan_alloc(p, off, &mem);
     if (rc) {               // no room: the byte rows run, from now on (no call asks again)
