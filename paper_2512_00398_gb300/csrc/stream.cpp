@@ -629,7 +629,7 @@ int hp_stream_get_stats(hp_stream* s, hp_stream_stats* out) {
     out->max_batch = s->max_batch;
     for (const BeamSlot& b : s->slots) out->admitted += b.beam >= 0;
     out->waiting = (int32_t)s->wait_q.size();
-    out->device_bytes = (int64_t)(s->arena_bytes + s->plan->tables_bytes);
+    out->device_bytes = (int64_t)(s->arena_bytes + s->plan->tables_bytes + s->plan->ptables_bytes);
     out->tail_samples = s->H;
     out->max_batch_seen = s->max_batch_seen;
     out->device_allocs = (s->arena ? 1 : 0) + s->plan->device_allocs;
