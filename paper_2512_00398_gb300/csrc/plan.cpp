@@ -838,6 +838,15 @@ int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cuda
     return HP_OK;
 }
 
+void drop_patterns(hp_plan* p) {
+    cudaDeviceSynchronize();
+    plan_free(p, p->ptables, p->ptables_bytes);
+    p->ptables = nullptr;
+    p->ptables_bytes = 0;
+    p->ptiling = DedispTiling();
+    p->pat_estimate = -1;
+}
+
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
                    int64_t out_pitch, int64_t nout, int njobs) {
     DedispJob J;

@@ -156,6 +156,8 @@ double estimate_patterns(const hp_plan* p);
 // estimated to be faster with them and s is not being captured (nothing can be
 // allocated then; the byte rows run).
 int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s);
+// Give the pattern-row tables back: the byte rows run from now on.
+void drop_patterns(hp_plan* p);
 // Append the tiles of every part, whose indices count from its own tables (left empty).
 void append_tiling(std::vector<DedispTiling>& parts, DedispTiling* T);
 // Estimated SM cycles of the byte-row kernel for `sums` (trial, channel, sample) sums.

@@ -509,17 +509,37 @@ int hp_stream_open(hp_stream** out, const hp_plan* tmpl, const hp_stream_config*
     rc = prepare_patterns(p, s->G + p->wmax - 1, L.xt_pitch, mb, nullptr);
     if (rc) { release(s); return rc; }
     if (cfg->hbm_budget > 0) {
-        const int64_t avail = cfg->hbm_budget - (int64_t)(p->tables_bytes + p->ptables_bytes);
-        const int64_t step1 = (int64_t)(s->ws_bytes + s->cand_dev_bytes);
-        while (mb >= 1 && mb * step1 + (int64_t)s->beam_bytes > avail) --mb;
-        if (mb < 1) { release(s); return HP_ERR_OOM; }
-        slots = (int)std::min<int64_t>(cfg->nbeams, (avail - mb * step1) / (int64_t)s->beam_bytes);
-        mb = std::min(mb, slots);
+        // step and beam slots beside `tables` bytes (none: {0, 0})
+        auto fit = [&](size_t tables) {
+            const int64_t avail = cfg->hbm_budget - (int64_t)tables;
+            const int64_t step1 = (int64_t)(s->ws_bytes + s->cand_dev_bytes);
+            int m = mb;
+            while (m >= 1 && m * step1 + (int64_t)s->beam_bytes > avail) --m;
+            if (m < 1) return std::make_pair(0, 0);
+            const int n = (int)std::min<int64_t>(cfg->nbeams, (avail - m * step1) / (int64_t)s->beam_bytes);
+            return std::make_pair(std::min(m, n), n);
+        };
+        std::pair<int, int> held = fit(p->tables_bytes + p->ptables_bytes);
+        if (p->ptables) {
+            // slots come before the pattern rows, which the byte rows can stand in for
+            const std::pair<int, int> rows = fit(p->tables_bytes);
+            if (rows.first > held.first || rows.second > held.second) {
+                drop_patterns(p);
+                held = rows;
+            }
+        }
+        if (held.first < 1) { release(s); return HP_ERR_OOM; }
+        mb = held.first;
+        slots = held.second;
     }
     s->max_batch = mb;
     s->beam_slots = slots;
     s->arena_bytes = (size_t)mb * (s->ws_bytes + s->cand_dev_bytes) + (size_t)slots * s->beam_bytes;
     rc = check_cuda(cudaMalloc(&s->arena, s->arena_bytes));
+    if (rc == HP_ERR_OOM && p->ptables) {
+        drop_patterns(p);
+        rc = check_cuda(cudaMalloc(&s->arena, s->arena_bytes));
+    }
     if (rc) { s->arena = nullptr; release(s); return rc; }
     uint8_t* a = s->arena;
     for (int j = 0; j < mb; ++j) {

@@ -1,5 +1,6 @@
 """Device memory of a stream whose plan takes the pattern rows: device_bytes counts their
-tables, so a budget of that many bytes holds the same stream again."""
+tables, so a budget of that many bytes holds the same stream again; a budget without room
+for them holds the same slots, on byte rows."""
 import numpy as np
 import pytest
 
@@ -32,3 +33,31 @@ def test_device_bytes_reopen_the_stream(hp, plan):                    # noqa: F8
     got, st = _open(hp, plan, hbm_budget=want[2])
     st.close()
     assert got == want
+
+
+def test_slots_come_before_the_pattern_tables(hp, plan):              # noqa: F811
+    import torch
+    want, st = _open(hp, plan)
+    st.close()
+    got, st = _open(hp, plan, hbm_budget=want[2] - 1)
+    assert got[:2] == want[:2] and got[2] < want[2]
+    # two gulps of every beam: the whole file's window of each is as the search's own
+    n = 2 * G
+    rng = np.random.Generator(np.random.PCG64(3))
+    x = [rng.integers(0, 40, size=(n, NCH), dtype=np.uint8) for _ in range(NB)]
+    for b in range(NB):
+        x[b][3000 + 100 * b:3004 + 100 * b] += 90
+        for g in range(2):
+            st.push(b, x[b][g * G:(g + 1) * G])
+    found = {}
+    while len(found) < 2 * NB:
+        info, c = st.poll(timeout_ms=60000)
+        assert info["status"] == hp.HP_OK
+        found[info["beam"], info["gulp_index"]] = c
+    st.close()
+    for b in range(NB):
+        # the first gulp's window starts at 0 and its series is the file's
+        got = found[b, 0]
+        want = hp.search(plan, torch.from_numpy(x[b][:G]).cuda())
+        near = lambda c: c[np.abs(c["sample"] - 3000 - 100 * b) < 8]   # noqa: E731
+        assert len(near(want)) > 0 and np.array_equal(near(got), near(want))
