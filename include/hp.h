@@ -360,6 +360,13 @@ typedef struct {
  * never reset). */
 int hp_plan_stats(hp_plan* plan, hp_stats* out, int reset);
 
+/* The kernel that the plan's last dedispersion launch was (hp_search, hp_dedisperse,
+ * hp_plan_autotune, or a batch's eager or captured call; the sums are the same):
+ * 0 byte rows, 1 pattern rows, k > 1 pattern rows whose last time tiles, or all of a
+ * short input's, were shared by k blocks each.  *kernel is host memory.
+ * HP_ERR_INVALID_ARG before the first one. */
+int hp_plan_dedisp_kernel(const hp_plan* plan, int* kernel);
+
 /* Candidate merging that allocates nothing (the paper has no counterpart).
  * Some callers cannot allocate device memory when they merge: a real-time
  * pipeline that forbids allocation after start-up (cudaMalloc can block and can

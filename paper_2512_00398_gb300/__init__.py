@@ -157,6 +157,13 @@ class Plan:
               "hp_plan_workspace_bytes")
         return int(v.value)
 
+    def dedisp_kernel(self) -> int:
+        """The kernel of the plan's last dedispersion launch: 0 byte rows, 1 pattern
+        rows, k > 1 pattern rows with tiles shared by k blocks each."""
+        v = C.c_int()
+        check(lib().hp_plan_dedisp_kernel(self.handle, C.byref(v)), "hp_plan_dedisp_kernel")
+        return int(v.value)
+
     def bind_workspace(self, nsamps: int, device=None):
         """Allocate the scratch for inputs of ``nsamps`` samples as a torch
         tensor and bind it, so the library itself allocates nothing."""

@@ -898,6 +898,12 @@ int split_tail(const hp_plan* p, DedispBatch* b, cudaStream_t s) {
                                         (size_t)p->ndm(), s));
 }
 
+int launched_kernel(const DedispBatch& b) {
+    int64_t k = 0;
+    for (int j = 0; j < b.njobs; ++j) k = std::max(k, b.jobs[j].pattern);
+    return (int)k;
+}
+
 // The dedispersion of the plan's own series also writes the second remedian
 // level (median baseline with at least two levels, direct dedispersion: the
 // layout holds the buffer only then), and the search starts from it.
@@ -945,6 +951,7 @@ int run_subband(hp_plan* p, const Layout& L, uint8_t* ws, int32_t* out, int64_t 
         stage_end(p, HP_STAGE_DEDISP, ti, s);
         if (rc) return rc;
         ++p->launches;
+        p->last_kernel = 0;
         SubbandArgs a;
         a.B = B;
         a.bpitch = L.sb_pitch;
@@ -1005,7 +1012,10 @@ int run_dedisp(hp_plan* p, const uint8_t* fb, int64_t nsamps, const Layout& L, u
     rc = split_tail(p, &B, s);
     if (!rc) rc = check_cuda(launch_dedisp(p->dedisp_cfg, B, p->status, p->timeout_ns, s));
     stage_end(p, HP_STAGE_DEDISP, ti, s);
-    if (!rc) ++p->launches;
+    if (!rc) {
+        ++p->launches;
+        p->last_kernel = launched_kernel(B);
+    }
     return rc;
 }
 
@@ -1320,6 +1330,7 @@ int batch_enqueue(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
             rc = split_tail(p, &db, s);
             if (!rc) rc = check_cuda(launch_dedisp(b->cfg, db, p->status, p->timeout_ns, s));
             if (rc) return rc;
+            p->last_kernel = launched_kernel(db);
             ++k;
         }
         rc = check_cuda(cudaEventRecord(b->dd_done[i], s));
@@ -1778,6 +1789,12 @@ int hp_plan_stats(hp_plan* p, hp_stats* out, int reset) {
     out->kernel_launches = p->launches;
     out->device_allocs = p->device_allocs;
     if (reset) p->launches = 0;
+    return HP_OK;
+}
+
+int hp_plan_dedisp_kernel(const hp_plan* p, int* kernel) {
+    if (!p || !kernel || p->last_kernel < 0) return HP_ERR_INVALID_ARG;
+    *kernel = p->last_kernel;
     return HP_OK;
 }
 

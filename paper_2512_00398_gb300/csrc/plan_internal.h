@@ -90,6 +90,7 @@ struct hp_plan {
     void* ptables = nullptr;
     size_t ptables_bytes = 0;
     int sm_count = 148;
+    int last_kernel = -1;              // hp_plan_dedisp_kernel
 
     // device state
     int device = -1;
@@ -156,6 +157,8 @@ double estimate_patterns(const hp_plan* p);
 // estimated to be faster with them and s is not being captured (nothing can be
 // allocated then; the byte rows run).
 int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s);
+// The kernel of a dedispersion launch, as hp_plan_dedisp_kernel reports it.
+int launched_kernel(const DedispBatch& b);
 // Give the pattern-row tables back: the byte rows run from now on.
 void drop_patterns(hp_plan* p);
 // Append the tiles of every part, whose indices count from its own tables (left empty).
