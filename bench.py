@@ -332,6 +332,7 @@ def run_ours(args):
     if st != hp.HP_OK:
         raise hp.HPError(st, "timed region")
     stats = hp.hp_plan_stats(plan, reset=True)
+    patterns = plan.dedisp_kernel() > 0       # the timed searches' dedispersion kernel
     # the same search with the RFI stage on (two more steps, not part of `value`)
     plan.set_param("rfi", 1)
     for _ in range(3):
@@ -459,9 +460,8 @@ def run_ours(args):
         peak_adds = 2.0 * peaks["int_add_ops_per_s"]
         achieved = adds / (dd_ms * 1e-3)
         cfg = int(plan.get_param("dedisp_config"))
-        # the default tile shape's plans take pattern rows (sums of up to four channels
-        # shared between trials): fewer additions than the byte-adds counted here
-        patterns = cfg == 17 and int(plan.get_param("fuse_levels")) == 0
+        # (pattern rows, sums of up to four channels shared between trials, need fewer
+        # additions than the byte-adds counted here)
         traffic = dedisp_traffic(w, cfg, patterns)
         alg_bytes = float(o.nchans) * o.nsamps + 4.0 * w.ndm * nout
         hbm_peak = measured_hbm_gbs()
