@@ -1271,6 +1271,21 @@ int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
     return HP_OK;
 }
 
+// The direct dedispersion of one file of a batch.
+int batch_dedisp(hp_batch* b, int i, const Layout& L, uint8_t* ws, bool fuse, cudaStream_t s) {
+    hp_plan* p = b->plans[i];
+    DedispBatch db;
+    std::memset(&db, 0, sizeof(db));
+    db.njobs = 1;
+    db.jobs[0] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout);
+    if (fuse) fuse_levels(db.jobs[0], L, ws);
+    db.prefix[1] = (int64_t)db.jobs[0].ntt * db.jobs[0].ndt;
+    int rc = split_tail(p, &db, s);
+    if (!rc) rc = check_cuda(launch_dedisp(b->cfg, db, p->status, p->timeout_ns, s));
+    if (!rc) p->last_kernel = launched_kernel(db);
+    return rc;
+}
+
 // Enqueue the whole batch on s: one transpose launch, one dedispersion launch
 // over every file's tiles, then per file search + merge on a side stream.
 // One call of a batch: one transpose launch over every file; then the files'
@@ -1321,16 +1336,8 @@ int batch_enqueue(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
             if (rc) return rc;
             k += p->launches - before;
         } else {
-            DedispBatch db;
-            std::memset(&db, 0, sizeof(db));
-            db.njobs = 1;
-            db.jobs[0] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout);
-            fuse_levels(db.jobs[0], L, ws);
-            db.prefix[1] = (int64_t)db.jobs[0].ntt * db.jobs[0].ndt;
-            rc = split_tail(p, &db, s);
-            if (!rc) rc = check_cuda(launch_dedisp(b->cfg, db, p->status, p->timeout_ns, s));
+            rc = batch_dedisp(b, i, L, ws, true, s);
             if (rc) return rc;
-            p->last_kernel = launched_kernel(db);
             ++k;
         }
         rc = check_cuda(cudaEventRecord(b->dd_done[i], s));
@@ -1943,9 +1950,7 @@ int hp_batch_autotune(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsa
         if (rc) break;
         TransposeBatch tb;
         std::memset(&tb, 0, sizeof(tb));
-        DedispBatch db;
-        std::memset(&db, 0, sizeof(db));
-        tb.njobs = db.njobs = n;
+        tb.njobs = n;
         bool reach = true;
         for (int i = 0; i < n; ++i) {
             hp_plan* p = b->plans[i];
@@ -1953,20 +1958,20 @@ int hp_batch_autotune(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsa
             reach = reach && reach_ok(p, L.nout, L.xt_pitch);
             tb.jobs[i] = make_transpose_job(fbs[i], nsamps[i], p->nchans, wss[i] + L.xt, L.xt_pitch);
             tb.prefix[i + 1] = tb.prefix[i] + tb.jobs[i].ttiles * tb.jobs[i].ctiles;
-            db.jobs[i] = make_job(p, wss[i] + L.xt, L.xt_pitch, (int32_t*)(wss[i] + L.D), L.dpitch,
-                                  L.nout);
-            db.prefix[i + 1] = db.prefix[i] + (int64_t)db.jobs[i].ntt * db.jobs[i].ndt;
         }
         if (!reach) continue;          // this tile shape cannot stage these rows
-        hp_plan* p0 = b->plans[0];
+        // the launches that a search makes
+        auto pass = [&]() {
+            int r = check_cuda(launch_transpose_batch(tb, s));
+            for (int i = 0; i < n && !r; ++i) r = batch_dedisp(b, i, Ls[i], wss[i], false, s);
+            return r;
+        };
         if (!warm) {   // one untimed pass before the first timed one
-            rc = check_cuda(launch_transpose_batch(tb, s));
-            if (!rc) rc = check_cuda(launch_dedisp(c, db, p0->status, p0->timeout_ns, s));
+            rc = pass();
             warm = true;
         }
         if (!rc) rc = check_cuda(cudaEventRecord(e0, s));
-        if (!rc) rc = check_cuda(launch_transpose_batch(tb, s));
-        if (!rc) rc = check_cuda(launch_dedisp(c, db, p0->status, p0->timeout_ns, s));
+        if (!rc) rc = pass();
         if (!rc) rc = check_cuda(cudaEventRecord(e1, s));
         if (!rc) rc = check_cuda(cudaEventSynchronize(e1));
         float ms = 0.f;
