@@ -491,19 +491,7 @@ cudaError_t launch_dedisp(int cfg, const DedispBatch& b, int* status, uint64_t t
     int npat = 0;
     for (int j = 0; j < b.njobs; ++j) npat += b.jobs[j].pattern != 0;
     if (npat == b.njobs && npat > 0) return launch_dedisp_patterns(b, status, timeout_ns, s);
-    if (npat > 0) {
-        // jobs of both kernels: one launch of each
-        DedispBatch part[2];
-        std::memset(part, 0, sizeof(part));
-        for (int j = 0; j < b.njobs; ++j) {
-            DedispBatch& q = part[b.jobs[j].pattern != 0];
-            q.jobs[q.njobs] = b.jobs[j];
-            q.prefix[q.njobs + 1] = q.prefix[q.njobs] + (b.prefix[j + 1] - b.prefix[j]);
-            ++q.njobs;
-        }
-        const cudaError_t e = launch_dedisp(cfg, part[1], status, timeout_ns, s);
-        return e != cudaSuccess ? e : launch_dedisp(cfg, part[0], status, timeout_ns, s);
-    }
+    if (npat > 0) return cudaErrorInvalidValue;   // the jobs of a launch take one kernel
     const int sb = kDedispConfigs[cfg].stage_bytes;
     switch (cfg) {
         case 0: return run_dedisp_rows<2, 5, 8, 2, 6>(b, sb, status, timeout_ns, s);

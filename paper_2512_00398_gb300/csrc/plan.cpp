@@ -741,7 +741,7 @@ double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total,
     return best;
 }
 
-// Is a launch of njobs inputs of nout samples faster with pattern rows that take
+// Is a launch of njobs inputs (nout[j] samples) faster with pattern rows that take
 // `cycles` per time tile?  Both kernels keep one block per SM, so the one whose last
 // wave ends first, by the estimated cycles of its blocks: the pattern rows' larger
 // tiles (24 trials x 2048 samples against 15 x 2176) lose on short inputs, where a
@@ -751,26 +751,33 @@ double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total,
 // trials, 4000 samples 0.833 ms by byte rows, 0.256 by parts of pattern rows; 2048
 // channels, 200 trials, 8192 samples 0.421 and 0.160.  There the tables must earn more
 // (1.25): they cost the plan's first call 2 to 5 ms.
-bool patterns_pay(const hp_plan* p, double cycles, int64_t nout, int njobs) {
+bool patterns_pay(const hp_plan* p, double cycles, const int64_t* nout, int njobs) {
     // the default tile shape of direct dedispersion, without fused remedian levels
     if (p->dedisp_cfg != kDefaultDedispConfig || p->sb_chans > 0 || p->fuse_levels) return false;
-    if (cycles <= 0 || nout <= 0) return false;
+    if (cycles <= 0 || njobs < 1) return false;
     const DedispTiling& T = p->tiling;
     const int64_t nt = (int64_t)T.tiles.size(), nq = ceil_div(p->ndm(), kPatBD);
+    int64_t qcols = 0, tcols = 0;
+    for (int j = 0; j < njobs; ++j) {
+        if (nout[j] <= 0) return false;
+        qcols += ceil_div(nout[j], kPatBT);
+        tcols += ceil_div(nout[j], T.BT);
+    }
     const double tile = cycles / (double)nq;
-    const int64_t ntt = ceil_div(nout, kPatBT);
-    const double q = (double)ceil_div(ntt * nq * njobs, p->sm_count) * tile;
-    const double t = (double)ceil_div(ceil_div(nout, T.BT) * nt * njobs, p->sm_count) *
+    const double q = (double)ceil_div(qcols * nq, p->sm_count) * tile;
+    const double t = (double)ceil_div(tcols * nt, p->sm_count) *
                      byte_row_cycles((double)T.BD * p->nchans * T.BT);
     int cols, parts;
-    return q * 1.03 < t ||
-           pattern_waves(p, cycles, nq, ntt * nq * njobs, (int)ntt, &cols, &parts) * tile * 1.25 < t;
+    return q * 1.03 < t || pattern_waves(p, cycles, nq, qcols * nq, (int)ceil_div(nout[njobs - 1], kPatBT),
+                                         &cols, &parts) * tile * 1.25 < t;
 }
 
-bool use_patterns(const hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs) {
+bool use_patterns(const hp_plan* p, const int64_t* nout, const int64_t* xt_pitch, int njobs) {
     const DedispTiling& Q = p->ptiling;
-    return p->ptables && (ceil_div(nout, Q.BT) - 1) * Q.BT + Q.max_reach <= xt_pitch &&
-           patterns_pay(p, Q.cycles, nout, njobs);
+    if (!p->ptables) return false;
+    for (int j = 0; j < njobs; ++j)
+        if ((ceil_div(nout[j], Q.BT) - 1) * Q.BT + Q.max_reach > xt_pitch[j]) return false;
+    return patterns_pay(p, Q.cycles, nout, njobs);
 }
 
 // While it lives, this thread's allocations and copies are allowed beside another
@@ -782,12 +789,14 @@ struct BesideCaptures {
     ~BesideCaptures() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s) {
+int prepare_patterns(hp_plan* p, int64_t nout, int njobs, cudaStream_t s) {
     if (p->ptables || p->pat_estimate < 0 || p->dedisp_cfg != kDefaultDedispConfig ||
         p->sb_chans > 0 || p->fuse_levels)
         return HP_OK;
     if (p->pat_estimate == 0) p->pat_estimate = estimate_patterns(p);
-    if (!patterns_pay(p, p->pat_estimate, nout, njobs)) return HP_OK;
+    int64_t nouts[kMaxJobs];
+    std::fill_n(nouts, kMaxJobs, nout);
+    if (!patterns_pay(p, p->pat_estimate, nouts, std::min(njobs, kMaxJobs))) return HP_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (check_cuda(cudaStreamIsCapturing(s, &cap)) || cap != cudaStreamCaptureStatusNone)
         return HP_OK;
@@ -848,9 +857,8 @@ void drop_patterns(hp_plan* p) {
 }
 
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
-                   int64_t out_pitch, int64_t nout, int njobs) {
+                   int64_t out_pitch, int64_t nout, bool pat) {
     DedispJob J;
-    const bool pat = use_patterns(p, nout, xt_pitch, njobs);
     const DedispTiling& T = pat ? p->ptiling : p->tiling;
     J.xt = xt;
     J.xt_pitch = xt_pitch;
@@ -940,7 +948,7 @@ int run_subband(hp_plan* p, const Layout& L, uint8_t* ws, int32_t* out, int64_t 
         db.njobs = n;
         for (int k = 0; k < n; ++k) {
             DedispJob J = make_job(p, ws + L.xt, L.xt_pitch, B + (size_t)k * rows * L.sb_pitch,
-                                   L.sb_pitch, L.sb_len);
+                                   L.sb_pitch, L.sb_len, false);
             J.tiles = p->d_tiles + (c0 + k);
             J.ndt = 1;
             db.jobs[k] = J;
@@ -998,13 +1006,13 @@ int run_dedisp(hp_plan* p, const uint8_t* fb, int64_t nsamps, const Layout& L, u
         if (rc) return rc;
     }
     if (p->sb_chans > 0) return run_subband(p, L, ws, out, out_pitch, s);
-    rc = prepare_patterns(p, nout, xt_pitch, 1, s);
+    rc = prepare_patterns(p, nout, 1, s);
     if (rc) return rc;
     DedispBatch B;   // copied into the kernel parameters at launch
     std::memset(&B, 0, sizeof(B));
     B.njobs = 1;
     if (!reach_ok(p, nout, xt_pitch)) return HP_ERR_INVALID_ARG;
-    B.jobs[0] = make_job(p, xt, xt_pitch, out, out_pitch, nout);
+    B.jobs[0] = make_job(p, xt, xt_pitch, out, out_pitch, nout, use_patterns(p, &nout, &xt_pitch, 1));
     if (own_series) fuse_levels(B.jobs[0], L, ws);
     B.prefix[0] = 0;
     B.prefix[1] = (int64_t)B.jobs[0].ntt * B.jobs[0].ndt;
@@ -1263,7 +1271,7 @@ int batch_prepare(hp_batch* b, const uint8_t* const* fbs, const int64_t* nsamps,
         rc = ensure_device_tables(p, s);
         if (rc) return rc;
         (*layouts)[i] = make_layout(p, nsamps[i], true);
-        rc = prepare_patterns(p, (*layouts)[i].nout, (*layouts)[i].xt_pitch, 1, s);
+        rc = prepare_patterns(p, (*layouts)[i].nout, 1, s);
         if (rc) return rc;
         rc = ensure_workspace(p, (*layouts)[i].total, &(*wss)[i]);
         if (rc) return rc;
@@ -1277,7 +1285,8 @@ int batch_dedisp(hp_batch* b, int i, const Layout& L, uint8_t* ws, bool fuse, cu
     DedispBatch db;
     std::memset(&db, 0, sizeof(db));
     db.njobs = 1;
-    db.jobs[0] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout);
+    db.jobs[0] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout,
+                          use_patterns(p, &L.nout, &L.xt_pitch, 1));
     if (fuse) fuse_levels(db.jobs[0], L, ws);
     db.prefix[1] = (int64_t)db.jobs[0].ntt * db.jobs[0].ndt;
     int rc = split_tail(p, &db, s);

@@ -156,7 +156,10 @@ double estimate_patterns(const hp_plan* p);
 // Build the pattern-row tables if a launch of njobs inputs of nout samples is
 // estimated to be faster with them and s is not being captured (nothing can be
 // allocated then; the byte rows run).
-int prepare_patterns(hp_plan* p, int64_t nout, int64_t xt_pitch, int njobs, cudaStream_t s);
+int prepare_patterns(hp_plan* p, int64_t nout, int njobs, cudaStream_t s);
+// Does a launch of njobs inputs, nout[j] samples from rows of xt_pitch[j] bytes, take the
+// pattern rows?  (They are there and estimated to be faster.)
+bool use_patterns(const hp_plan* p, const int64_t* nout, const int64_t* xt_pitch, int njobs);
 // The kernel of a dedispersion launch, as hp_plan_dedisp_kernel reports it.
 int launched_kernel(const DedispBatch& b);
 // Give the pattern-row tables back: the byte rows run from now on.
@@ -175,10 +178,10 @@ bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch);
 // blocks each where that fills a last wave that would be nearly empty (zeroes their
 // part of the output on s).
 int split_tail(const hp_plan* p, DedispBatch* b, cudaStream_t s);
-// One job of a launch of about `njobs` such jobs (the choice between the byte-row
-// and the pattern-row kernel depends on how many blocks the launch has).
+// One job of a launch, with the tables of the pattern rows or of the byte rows (one
+// kernel for all jobs of a launch, use_patterns).
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
-                   int64_t out_pitch, int64_t nout, int njobs = 1);
+                   int64_t out_pitch, int64_t nout, bool pat);
 // Stages 1 and 2 of the sub-band variant on the transposed input at ws + L.xt.
 int run_subband(hp_plan* p, const Layout& L, uint8_t* ws, int32_t* out, int64_t out_pitch,
                 cudaStream_t s);

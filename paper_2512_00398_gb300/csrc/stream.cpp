@@ -306,16 +306,26 @@ int enqueue_step(hp_stream* s, Step* st) {
         J.ring_slots = s->R;
         tb.jobs[j] = J;
         tb.prefix[j + 1] = tb.prefix[j] + J.ttiles * J.ctiles;
-        if (p->sb_chans <= 0) {   // the sub-band variant runs its own two stages per gulp
-            if (!reach_ok(p, L.nout, L.xt_pitch)) return HP_ERR_INVALID_ARG;
-            db.jobs[j] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout,
-                                  (int)st->items.size());
-            fuse_levels(db.jobs[j], L, ws);
-            db.prefix[j + 1] = db.prefix[j] + (int64_t)db.jobs[j].ntt * db.jobs[j].ndt;
-        }
         work.push_back(&it);
     }
     const int n = (int)work.size();
+    if (n > 0 && p->sb_chans <= 0) {   // (the sub-band variant runs its own two stages per gulp)
+        // one kernel for all of a step's gulps, a beam's shorter first ones among them
+        std::vector<int64_t> nout, pitch;
+        for (const Layout& L : Ls) {
+            if (!reach_ok(p, L.nout, L.xt_pitch)) return HP_ERR_INVALID_ARG;
+            nout.push_back(L.nout);
+            pitch.push_back(L.xt_pitch);
+        }
+        const bool pat = use_patterns(p, nout.data(), pitch.data(), n);
+        for (int j = 0; j < n; ++j) {
+            const Layout& L = Ls[j];
+            uint8_t* ws = s->ws[j];
+            db.jobs[j] = make_job(p, ws + L.xt, L.xt_pitch, (int32_t*)(ws + L.D), L.dpitch, L.nout, pat);
+            fuse_levels(db.jobs[j], L, ws);
+            db.prefix[j + 1] = db.prefix[j] + (int64_t)db.jobs[j].ntt * db.jobs[j].ndt;
+        }
+    }
     if (n > 0) {
         tb.njobs = n;
         db.njobs = p->sb_chans > 0 ? 0 : n;
@@ -506,7 +516,7 @@ int hp_stream_open(hp_stream** out, const hp_plan* tmpl, const hp_stream_config*
     mb = std::min(mb, cfg->nbeams);
     int slots = cfg->nbeams;
     // (a gulp's window and the look-ahead of the widest boxcar)
-    rc = prepare_patterns(p, s->G + p->wmax - 1, L.xt_pitch, mb, nullptr);
+    rc = prepare_patterns(p, s->G + p->wmax - 1, mb, nullptr);
     if (rc) { release(s); return rc; }
     if (cfg->hbm_budget > 0) {
         // step and beam slots beside `tables` bytes (none: {0, 0})
