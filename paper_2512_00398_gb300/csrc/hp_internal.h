@@ -323,6 +323,7 @@ struct MergeArgs {
     int dm_tol;
     int64_t t_gap;
     int w_tol;
+    int64_t small_max;         // longest list that one block takes (launch_merge)
     // scratch
     uint64_t* keys[2];
     int64_t* vals[2];

@@ -28,10 +28,11 @@
 //      correctly rounded operations (ties: smallest key).
 //   4. roots are compacted in index order with a device-wide scan.
 //
-// A list of at most 2048 candidates, the usual one, goes through all of it in one
-// block's shared memory (merge_small_kernel); the kernels of the general path then
-// find nothing to do.  The host cannot know the count, so they are launched all the
-// same: few of them, and each starting while the one before it drains.
+// A list of at most 1024 candidates (fewer with a large dm_tol: small_list), the usual
+// one, goes through all of it in one block's shared memory (merge_small_kernel); the
+// kernels of the general path then find nothing to do.  The host cannot know the count,
+// so they are launched all the same: few of them, and each starting while the one before
+// it drains.
 //
 // Measured, against one union per touching pair, two-way passes and 21 launches: 215
 // candidates (tiny search) 44 us, before 165; 25 855 (FAST-like file) 146, before
@@ -633,12 +634,23 @@ __global__ void __launch_bounds__(kScanBlock) scatter_kernel(MergeArgs a) {
     }
 }
 
-// The whole merge of at most kSmall candidates in one block's shared memory; it
-// leaves *n_clamped = -1 to the general path's kernels.  Longer lists: their length,
+// The whole merge of at most kSmall candidates, one per thread, in one block's shared
+// memory; it leaves *n_clamped = -1 to the general path's kernels.  Longer lists: their length,
 // the counters, the status.  What bounds it is the chain of barriers and
 // shared-memory latencies of the sort (a list of 256 takes 3 block barriers, of
-// 2048 18) and the friend scans.
-constexpr int kSmall = kSortChunk;
+// 1024 13) and the links.
+constexpr int kSmall = 1024;
+
+// The longest list for one block: up to here it is faster than the general path's
+// kernels on all 152 SMs.  Links to the next dm_tol trials grow with dm_tol, and one SM
+// makes them.  One block and general path, us, lists with clusters and dense ones (those
+// of 2000 at two candidates a thread):
+//    defaults:           1024  54 and  82,  44 and 68       2000  101 and  86,   79 and  71
+//    friend scans:       1024  78 and 119, 482 and 480      2000  142 and 124, 1392 and 925
+//    dm_tol 16, scans:    512 311 and 338, 508 and 622      1024  394 and 351,  986 and 1032
+//    dm_tol 64, scans:    128 377 and 321, 146 and 339       512  863 and 581,  510 and 798
+//    dm_tol 64:           128 108 and 163,  63 and 79       1024  615 and 291,  258 and 122
+int64_t small_list(int dm_tol) { return std::max(32, std::min(kSmall, 8192 / std::max(dm_tol, 1))); }
 
 struct SmallState {
     uint64_t key[kSmall];
@@ -657,79 +669,68 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(MergeArgs a) {
     const int64_t nr = *a.nraw;
     const int64_t nc = nr < a.cap ? nr : a.cap;
     if (t == 0) {
-        *a.n_clamped = nc <= kSmall ? -1 : nc;
+        *a.n_clamped = nc <= a.small_max ? -1 : nc;
         if (nr > a.cap) latch_status(a.status, HP_ERR_CAND_OVERFLOW);
-        if (nc > kSmall)
+        if (nc > a.small_max)
             for (int i = 0; i < 4; ++i) a.scan[i] = 0;
     }
-    if (nc > kSmall) return;
+    if (nc > a.small_max) return;
     const int n = nc > 0 ? (int)nc : 0;
     int size = 64;
     while (size < n) size <<= 1;
-    for (int i = t; i < size; i += 1024) {
-        s.key[i] = kPad;
-        s.val[i] = 0;
-        if (i < n) {
-            const hp_raw_cand c = a.raw[i];
-            s.key[i] = cand_key(c);
-            s.val[i] = c.S;
+    if (t < size) {
+        s.key[t] = kPad;
+        s.val[t] = 0;
+        if (t < n) {
+            const hp_raw_cand c = a.raw[t];
+            s.key[t] = cand_key(c);
+            s.val[t] = c.S;
         }
-        s.best[i] = 0;
-        s.members[i] = 0;
-        s.dm_lo[i] = INT_MAX;
-        s.dm_hi[i] = INT_MIN;
-        s.t_lo[i] = ~0ull;
+        s.best[t] = 0;
+        s.members[t] = 0;
+        s.dm_lo[t] = INT_MAX;
+        s.dm_hi[t] = INT_MIN;
+        s.t_lo[t] = ~0ull;
     }
     if (t < a.nw) s.widths[t] = a.widths[t];
     __syncthreads();
     bitonic_sort(s.key, s.val, size);
     __syncthreads();
     if (any_window(a)) {
-        // components (two neighbouring entries per thread): the running maxima in
-        // t_hi, the heads in parent
-        uint64_t key[2] = {}, w[2] = {}, total;
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-            if (2 * t + e < n) {
-                key[e] = s.key[2 * t + e];
-                w[e] = end_word(key[e], s.widths);
-            }
-        const uint64_t b0 = block_max_exclusive(max(w[0], w[1]), s.warp_max, &total);
-        const uint64_t b1 = max(b0, w[0]);
-        const bool h0 = 2 * t < n && (t == 0 || starts_component(key[0], b0, a.t_gap));
-        const bool h1 = 2 * t + 1 < n && starts_component(key[1], b1, a.t_gap);
-        const uint64_t m0 = h0 ? 2 * t + 1 : 0, m1 = h1 ? 2 * t + 2 : m0;
-        const uint64_t hb = block_max_exclusive(m1, s.warp_max, &total);
-        if (2 * t < n) {
-            s.t_hi[2 * t] = b1;
-            s.parent[2 * t] = s.rep[2 * t] = (int32_t)max(hb, m0) - 1;
-        }
-        if (2 * t + 1 < n) {
-            s.t_hi[2 * t + 1] = max(b1, w[1]);
-            s.parent[2 * t + 1] = s.rep[2 * t + 1] = (int32_t)max(hb, m1) - 1;
+        // components: the running maxima in t_hi, the heads in parent
+        const uint64_t key = t < n ? s.key[t] : 0;
+        const uint64_t w = t < n ? end_word(key, s.widths) : 0;
+        uint64_t total;
+        const uint64_t before = block_max_exclusive(w, s.warp_max, &total);
+        const bool head = t < n && (t == 0 || starts_component(key, before, a.t_gap));
+        const uint64_t mine = head ? t + 1 : 0;
+        const uint64_t h = max(mine, block_max_exclusive(mine, s.warp_max, &total));
+        if (t < n) {
+            s.t_hi[t] = max(before, w);
+            s.parent[t] = s.rep[t] = (int32_t)h - 1;
         }
         __syncthreads();
-        for (int i = t; i < n; i += 1024)
-            if (i + 1 == n || s.rep[i + 1] == i + 1)   // rep keeps the heads while parent changes
-                link_component(a, s.key, n, s.rep[i], i, [&](int64_t j) { return (uint64_t)s.t_hi[j]; },
-                               [&](int64_t j) { return (int64_t)s.rep[j]; }, s.parent, nullptr);
+        if (t < n && (t + 1 == n || s.rep[t + 1] == t + 1))   // rep keeps the heads while parent changes
+            link_component(a, s.key, n, s.rep[t], t, [&](int64_t j) { return (uint64_t)s.t_hi[j]; },
+                           [&](int64_t j) { return (int64_t)s.rep[j]; }, s.parent, nullptr);
     } else {
-        for (int i = t; i < n; i += 1024) s.parent[i] = i;
+        if (t < n) s.parent[t] = t;
         __syncthreads();
-        for (int i = t; i < n; i += 1024)
-            link_candidate(a, s.widths, s.key, n, i, s.parent, nullptr);
+        if (t < n) link_candidate(a, s.widths, s.key, n, t, s.parent, nullptr);
     }
     __syncthreads();
-    for (int i = t; i < n; i += 1024) {
-        s.rep[i] = INT_MAX;
-        s.t_hi[i] = 0;
+    if (t < n) {
+        s.rep[t] = INT_MAX;
+        s.t_hi[t] = 0;
     }
     __syncthreads();
-    for (int i = t; i < n; i += 1024) {
-        const int32_t r = uf_find(s.parent, i);
-        s.parent[i] = r;
-        const uint64_t k = s.key[i];
-        atomicMax(&s.best[r], (unsigned long long)__double_as_longlong(cand_snr(a, s.widths, k, s.val[i])));
+    const uint64_t k = t < n ? s.key[t] : 0;
+    const double snr = t < n ? cand_snr(a, s.widths, k, s.val[t]) : 0.0;
+    int32_t r = 0;
+    if (t < n) {
+        r = uf_find(s.parent, t);
+        s.parent[t] = r;
+        atomicMax(&s.best[r], (unsigned long long)__double_as_longlong(snr));
         atomicAdd(&s.members[r], 1);
         atomicMin(&s.dm_lo[r], key_dm(k));
         atomicMax(&s.dm_hi[r], key_dm(k));
@@ -738,35 +739,27 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(MergeArgs a) {
         atomicMax(&s.t_hi[r], ts + (unsigned long long)s.widths[key_width(k)]);
     }
     __syncthreads();
-    for (int i = t; i < n; i += 1024) {
-        const int32_t r = s.parent[i];
-        const double snr = cand_snr(a, s.widths, s.key[i], s.val[i]);
-        if ((unsigned long long)__double_as_longlong(snr) == s.best[r]) atomicMin(&s.rep[r], i);
-    }
+    if (t < n && (unsigned long long)__double_as_longlong(snr) == s.best[r]) atomicMin(&s.rep[r], t);
     __syncthreads();
-    int32_t done = 0;
-    for (int i0 = 0; i0 < n; i0 += 1024) {   // (block-uniform)
-        const int i = i0 + t;
-        const bool root = i < n && s.parent[i] == i;
-        int32_t total;
-        const int64_t slot = done + block_exclusive(root, s.warp_tot, &total);
-        done += total;
-        if (!root || slot >= a.out_cap) continue;
-        const int32_t rp = s.rep[i];
+    const bool root = t < n && r == t;
+    int32_t total;
+    const int64_t slot = block_exclusive(root, s.warp_tot, &total);
+    if (root && slot < a.out_cap) {
+        const int32_t rp = s.rep[t];
         const uint64_t kr = s.key[rp];
         hp_cand c;
         c.dm_idx = key_dm(kr);
         c.width_idx = key_width(kr);
         c.sample = key_sample(kr);
         c.snr = (float)cand_snr(a, s.widths, kr, s.val[rp]);
-        c.members = s.members[i];
-        c.dm_lo = s.dm_lo[i];
-        c.dm_hi = s.dm_hi[i];
-        c.t_lo = (int64_t)s.t_lo[i];
-        c.t_hi = (int64_t)s.t_hi[i];
+        c.members = s.members[t];
+        c.dm_lo = s.dm_lo[t];
+        c.dm_hi = s.dm_hi[t];
+        c.t_lo = (int64_t)s.t_lo[t];
+        c.t_hi = (int64_t)s.t_hi[t];
         a.out[slot] = c;
     }
-    if (t == 0) *a.out_count = done;
+    if (t == 0) *a.out_count = total;
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -798,7 +791,8 @@ std::atomic<int> g_wave[11];
 }  // namespace
 
 cudaError_t launch_merge(const MergeArgs& a_in, cudaStream_t s, int64_t* nlaunch) {
-    const MergeArgs a = a_in;
+    MergeArgs a = a_in;
+    a.small_max = small_list(a.dm_tol);
     if (a.cap <= 0) {
         return cudaMemsetAsync(a.out_count, 0, sizeof(int64_t), s);
     }
@@ -807,7 +801,7 @@ cudaError_t launch_merge(const MergeArgs& a_in, cudaStream_t s, int64_t* nlaunch
     if (e != cudaSuccess) return e;
     ++*nlaunch;
     e = launch_pdl(merge_small_kernel, 1, 1024, sizeof(SmallState), s, a);
-    if (e != cudaSuccess || a.cap <= kSmall) return e;
+    if (e != cudaSuccess || a.cap <= a.small_max) return e;
     const int64_t padded_cap = ceil_div(a.cap, kSortChunk) * kSortChunk;
     // grids of at most one resident wave; the kernels stride over the rest
     const int64_t g256 = ceil_div(padded_cap, 256);
