@@ -202,13 +202,24 @@ int hp_plan_max_delay(const hp_plan* plan, int32_t* max_delay);
 int hp_plan_workspace_bytes(const hp_plan* plan, int64_t nsamps, size_t* bytes);
 
 /* Give the plan a caller-owned device workspace (256-byte aligned, at least
- * hp_plan_workspace_bytes).  While bound, the plan allocates no scratch (its
- * constant tables, a few MB, are allocated once by the first search); the
+ * hp_plan_workspace_bytes).  While bound, the plan allocates no scratch, only
+ * its constant tables (hp_plan_prepare); the
  * caller keeps ownership and must keep it alive until the plan is destroyed
  * or another workspace is bound.  Passing NULL unbinds (the plan then
  * allocates its own scratch with cudaMalloc on demand, grow-only).  The size
  * depends on the raw capacity and baseline mode: query it after setting them. */
 int hp_plan_bind_workspace(hp_plan* plan, void* workspace_dev, size_t bytes);
+
+/* Build now what hp_search, hp_dedisperse or a batch with an input of nsamps samples
+ * would build at its first call, so that this call allocates and copies nothing and
+ * may be captured: the plan's scratch, unless a workspace is bound, and its constant
+ * tables.  There are two of these, each up to tens of MB (4096 channels, 1500 trials):
+ * those of the tile shape, built by the plan's first call, and with the default shape
+ * those of the pattern rows, built by the first call, which may be a later one, whose
+ * length makes them pay, and kept for every call after it.  Without them, while `stream` is captured
+ * and where their allocation is refused, the byte rows run instead (same sums).
+ * Waits for `stream`; HP_ERR_NSAMPS_TOO_SHORT as for hp_search. */
+int hp_plan_prepare(hp_plan* plan, int64_t nsamps, void* stream);
 
 /* ----------------------------------------------------------- the hot path */
 

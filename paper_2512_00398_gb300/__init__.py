@@ -157,6 +157,11 @@ class Plan:
               "hp_plan_workspace_bytes")
         return int(v.value)
 
+    def prepare(self, nsamps: int, stream=None):
+        """Build what the first search of ``nsamps`` samples would build (tables, and
+        scratch unless a workspace is bound), so that it allocates nothing and can be captured."""
+        check(lib().hp_plan_prepare(self.handle, int(nsamps), _stream_ptr(stream)), "hp_plan_prepare")
+
     def dedisp_kernel(self) -> int:
         """The kernel of the plan's last dedispersion launch: 0 byte rows, 1 pattern
         rows, k > 1 pattern rows with tiles shared by k blocks each."""

@@ -64,7 +64,8 @@ EXPORTS = ("hp_status_str", "hp_plan_create", "hp_plan_destroy", "hp_plan_set_pa
            "hp_batch_autotune", "hp_batch_search", "hp_batch_sync_status",
            "hp_batch_kernels_per_call", "hp_stream_open", "hp_stream_push", "hp_stream_end_beam",
            "hp_stream_poll", "hp_stream_get_stats", "hp_stream_close", "hp_plan_set_allocator", "hp_rfi_clean",
-           "hp_width_sigmas", "hp_plan_dedisp_kernel")
+           "hp_width_sigmas", "hp_plan_dedisp_kernel",
+           "hp_plan_prepare")
 
 ALLOC_FN = C.CFUNCTYPE(C.c_void_p, C.c_size_t, C.c_void_p)
 FREE_FN = C.CFUNCTYPE(None, C.c_void_p, C.c_size_t, C.c_void_p)
@@ -168,6 +169,7 @@ def lib() -> C.CDLL:
             L.hp_plan_set_allocator.argtypes = [vp, ALLOC_FN, FREE_FN, vp]
             L.hp_rfi_clean.argtypes = [vp, vp, i64, vp, vp, vp, vp, vp]
             L.hp_width_sigmas.argtypes = [vp, vp, vp, vp]
+            L.hp_plan_prepare.argtypes = [vp, i64, vp]
             L.hp_plan_dedisp_kernel.argtypes = [vp, C.POINTER(i32)]
             for name in EXPORTS:
                 if name != "hp_status_str":

@@ -1650,6 +1650,18 @@ int hp_plan_bind_workspace(hp_plan* p, void* ws, size_t bytes) {
     return HP_OK;
 }
 
+int hp_plan_prepare(hp_plan* p, int64_t nsamps, void* stream) {
+    int rc = validate_search_input(p, p, nsamps);   // (the plan stands for the input's pointer)
+    if (rc) return rc;
+    rc = ensure_device_tables(p, (cudaStream_t)stream);
+    if (rc) return rc;
+    const Layout L = make_layout(p, nsamps, true);
+    uint8_t* ws = nullptr;
+    rc = ensure_workspace(p, L.total, &ws);
+    if (rc) return rc;
+    return prepare_patterns(p, L.nout, 1, (cudaStream_t)stream);
+}
+
 int hp_rfi_clean(hp_plan* p, const uint8_t* fb, int64_t nsamps, void* stream, uint8_t* cleaned,
                  uint8_t* chan_flag, uint8_t* samp_flag, int32_t* chan_median) {
     if (!p || !fb || nsamps < 1 || nsamps >= kMaxSamples) return HP_ERR_INVALID_ARG;
