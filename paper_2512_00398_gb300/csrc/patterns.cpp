@@ -43,12 +43,30 @@ struct TileOut {
     bool ok = false;
 };
 
+// The tables of one tile.  They are built by a call that waits for them: trying the
+// pattern of the trial before first, a channel's delays side by side and one list of
+// items a stage instead of vectors in each took the first call of a plan of one tile x
+// 1024 channels from 1.82 to 1.22 ms, of 17 tiles from 7.87 to 6.48.
 struct TileBuilder {
     const hp_plan* p;
     int d0, nd;
     bool strict;    // bound the tables of a group from above instead of estimating them
 
-    int32_t delay(int j, int c) const { return p->delays[(size_t)(d0 + j) * p->nchans + c]; }
+    std::vector<int32_t> column;   // delays of the channels from col0 on, nd trials each
+    int col0;
+
+    // For channels [begin, end) of trials [d0, d0 + nd).
+    TileBuilder(const hp_plan* plan, int first, int n, bool strict_, int begin, int end)
+        : p(plan), d0(first), nd(n), strict(strict_), column((size_t)n * (end - begin)), col0(begin) {
+        for (int j = 0; j < n; ++j) {
+            const int32_t* row = &p->delays[(size_t)(d0 + j) * p->nchans];
+            for (int c = begin; c < end; ++c) column[(size_t)(c - begin) * n + j] = row[c];
+        }
+    }
+
+    // (ascending: the trials are)
+    const int32_t* delays(int c) const { return &column[(size_t)(c - col0) * nd]; }
+    int32_t delay(int j, int c) const { return delays(c)[j]; }
 
     // Estimated SM cycles of a group whose sets unpack `sets` chunks in all and put
     // `rows` chunks into rows; fitted to 1620 cycles per group (15 and 51 chunks) at
@@ -62,26 +80,21 @@ struct TileBuilder {
         g->n = n;
         g->pats.clear();
         g->of_trial.assign(nd, 0);
-        int32_t lo = delay(0, c);
+        size_t i = 0;
         for (int j = 0; j < nd; ++j) {
             Pattern q{};
             for (int k = 0; k < n; ++k) q.rel[k] = delay(j, c + k) - delay(j, c);
             q.lo = q.hi = delay(j, c);
-            lo = std::min(lo, q.lo);
-            size_t i = 0;
-            while (i < g->pats.size() && std::memcmp(g->pats[i].rel, q.rel, sizeof(q.rel))) ++i;
+            // (mostly the pattern of the trial before)
+            if (j == 0 || std::memcmp(g->pats[i].rel, q.rel, sizeof(q.rel)))
+                for (i = 0; i < g->pats.size() && std::memcmp(g->pats[i].rel, q.rel, sizeof(q.rel));) ++i;
             if (i == g->pats.size()) g->pats.push_back(q);
-            g->pats[i].lo = std::min(g->pats[i].lo, q.lo);
-            g->pats[i].hi = std::max(g->pats[i].hi, q.hi);
+            g->pats[i].hi = q.hi;
             g->of_trial[j] = (int)i;
         }
-        g->u0 = lo & ~3;
+        g->u0 = delay(0, c) & ~3;
         for (int k = 0; k < n; ++k) {
-            int32_t a = delay(0, c + k), b = a;
-            for (int j = 1; j < nd; ++j) {
-                a = std::min(a, delay(j, c + k));
-                b = std::max(b, delay(j, c + k));
-            }
+            const int32_t a = delay(0, c + k), b = delay(nd - 1, c + k);
             g->goff[k] = a & ~15;
             g->nwords[k] = (uint32_t)((b - g->goff[k] + kPatBT + 15) / 16 * 4);
         }
@@ -117,16 +130,35 @@ struct TileBuilder {
     // One item of a set: its form cost (instructions, about) orders the items.
     struct Item {
         PatItem d;
+        int row, cost;             // its first row in `Items::rows`
+    };
+    struct Items {
+        std::vector<Item> items;
         std::vector<PatRow> rows;
-        int cost;
+        size_t bytes() const { return items.size() * sizeof(PatItem) + rows.size() * sizeof(PatRow); }
+        void clear() {
+            items.clear();
+            rows.clear();
+        }
+        // Append those of another list.
+        void append(const Items& more) {
+            for (Item it : more.items) {
+                it.row += (int)rows.size();
+                items.push_back(it);
+            }
+            rows.insert(rows.end(), more.rows.begin(), more.rows.end());
+        }
     };
 
     // The items of a group whose rows start at byte `row` of the row buffer and
     // whose channels' windows start at chan_off in the raw buffer; org: per pattern
     // the row buffer's byte offset of its word 0.
     void make_items(const Group& g, const std::vector<int>& ord, const uint32_t* chan_off, uint32_t row,
-                    std::vector<Item>* items, std::vector<uint32_t>* org) const {
+                    Items* out, std::vector<uint32_t>* org) const {
+        out->clear();
         org->assign(g.pats.size(), 0);
+        struct Row { int kind, lo, n; uint32_t row; };
+        Row rows[kPatBD];
         for (size_t i = 0; i < ord.size();) {
             int32_t lo[kPatMaxGroup];
             const size_t e = set_end(g, ord, i, lo);
@@ -137,9 +169,7 @@ struct TileBuilder {
                 d.off[slot(g.n, k)] = chan_off[k] + (uint32_t)(lo[k] & ~3);
                 d.sel[slot(g.n, k)] = (uint16_t)(0x3210u + 0x1111u * (uint32_t)(lo[k] & 3));
             }
-            struct Row { int kind, lo, n; uint32_t row; };
-            std::vector<Row> rows;
-            int first = 1 << 30, last = 0;
+            int first = 1 << 30, last = 0, nrows = 0;
             for (; i < e; ++i) {
                 const Pattern& q = g.pats[ord[i]];
                 int shift[4] = {};
@@ -154,7 +184,7 @@ struct TileBuilder {
                 row += (uint32_t)r.n * kPatChunk * 4;
                 first = std::min(first, r.lo);
                 last = std::max(last, r.lo + r.n);
-                rows.push_back(r);
+                rows[nrows++] = r;
             }
             // items of kPatItem chunks from the first chunk that any pattern covers
             for (int c0 = first; c0 < last; c0 += kPatItem) {
@@ -162,74 +192,73 @@ struct TileBuilder {
                 it.d = d;
                 for (int k = 0; k < 4; ++k) it.d.off[k] += (uint32_t)(c0 * kPatChunk);
                 it.cost = 200;
-                for (const Row& r : rows) {
+                it.row = (int)out->rows.size();
+                for (int k = 0; k < nrows; ++k) {
+                    const Row& r = rows[k];
                     uint32_t put = 0;
                     for (int q = 0; q < kPatItem; ++q)
                         if (c0 + q >= r.lo && c0 + q < r.lo + r.n) put |= 1u << q;
                     if (put == 0) continue;
                     // (the item may start before the row; those chunks' stores are masked)
-                    it.rows.push_back(
+                    out->rows.push_back(
                         PatRow{r.row + (uint32_t)((c0 - r.lo + kPatItem - 1) * kPatChunk * 4),
                                (uint16_t)put, (uint16_t)r.kind});
                     it.cost += 32;
                 }
-                if (it.rows.empty()) continue;
-                it.d.nrows = (uint8_t)it.rows.size();
-                items->push_back(std::move(it));
+                it.d.nrows = (uint8_t)(out->rows.size() - (size_t)it.row);
+                if (it.d.nrows) out->items.push_back(it);
             }
         }
     }
 
-    static uint32_t items_bytes(const std::vector<Item>& items) {
-        uint32_t b = 0;
-        for (const Item& it : items) b += (uint32_t)(sizeof(PatItem) + it.rows.size() * sizeof(PatRow));
-        return b;
+    // The same items in another stage: windows and rows start so many bytes further on.
+    static void move_items(uint32_t raw, uint32_t row, Items* out, std::vector<uint32_t>* org) {
+        for (Item& it : out->items)
+            for (uint32_t& off : it.d.off) off += raw;
+        for (PatRow& r : out->rows) r.at += row;
+        for (uint32_t& o : *org) o += row;
     }
 
     // The cheapest cut of the channels [begin, nch) into groups of 1 .. kPatMaxGroup.
     bool cut(int begin, int nch, std::vector<uint8_t>* len, double* total) const {
         std::vector<double> best(nch + 1, 0.0);
         len->assign(nch, 0);
-        std::vector<int> cls(nd), next(nd);
-        std::vector<std::pair<int, int32_t>> keys;   // the patterns, by refinement
-        std::vector<int32_t> lo(nd), hi(nd);         // their ranges of first-channel delays
+        int cls[kPatBD];
+        uint64_t keys[kPatBD];             // the patterns, by refinement: class, relative delay
+        int32_t lo[kPatBD], hi[kPatBD];    // their ranges of first-channel delays
         for (int c = nch - 1; c >= begin; --c) {
             best[c] = 1e300;
-            std::fill(cls.begin(), cls.end(), 0);
-            int32_t u0 = delay(0, c);
-            for (int j = 1; j < nd; ++j) u0 = std::min(u0, delay(j, c));
-            u0 &= ~3;
+            std::fill(cls, cls + nd, 0);
+            const int32_t* first = delays(c);
+            const int32_t u0 = first[0] & ~3;
             uint32_t raw = 0;
             int32_t range[kPatMaxGroup];       // of each channel's shift
             for (int n = 1; n <= kPatMaxGroup && c + n <= nch; ++n) {
                 // refine the classes by the n-th channel
-                keys.clear();
-                int32_t a = delay(0, c + n - 1), b = a;
-                int32_t r_lo = a - delay(0, c), r_hi = r_lo;
+                const int32_t* nth = delays(c + n - 1);
+                const int32_t a = nth[0], b = nth[nd - 1];
+                int32_t r_lo = a - first[0], r_hi = r_lo;
+                int nkeys = 0, i = 0;
                 for (int j = 0; j < nd; ++j) {
-                    const int32_t base = delay(j, c), v = delay(j, c + n - 1);
-                    a = std::min(a, v);
-                    b = std::max(b, v);
-                    r_lo = std::min(r_lo, v - base);
-                    r_hi = std::max(r_hi, v - base);
-                    const std::pair<int, int32_t> key(cls[j], v - base);
-                    size_t i = 0;
-                    while (i < keys.size() && keys[i] != key) ++i;
-                    if (i == keys.size()) {
-                        keys.push_back(key);
-                        lo[i] = hi[i] = base;
+                    const int32_t rel = nth[j] - first[j];
+                    r_lo = std::min(r_lo, rel);
+                    r_hi = std::max(r_hi, rel);
+                    const uint64_t key = (uint64_t)cls[j] << 32 | (uint32_t)rel;
+                    if (j == 0 || keys[i] != key)   // (mostly that of the trial before)
+                        for (i = 0; i < nkeys && keys[i] != key;) ++i;
+                    if (i == nkeys) {
+                        keys[nkeys++] = key;
+                        lo[i] = first[j];
                     }
-                    lo[i] = std::min(lo[i], base);
-                    hi[i] = std::max(hi[i], base);
-                    next[j] = (int)i;
+                    hi[i] = first[j];
+                    cls[j] = i;
                 }
-                cls = next;
                 raw += (uint32_t)((b - (a & ~15) + kPatBT + 15) / 16 * 16);
                 int chunks = 0, span = 0;
-                for (size_t i = 0; i < keys.size(); ++i) {
+                for (int k = 0; k < nkeys; ++k) {
                     Pattern q{};
-                    q.lo = lo[i];
-                    q.hi = hi[i];
+                    q.lo = lo[k];
+                    q.hi = hi[k];
                     const int e = chunk_hi(q, u0);
                     chunks += e - chunk_lo(q, u0);
                     span = std::max(span, e);
@@ -240,10 +269,10 @@ struct TileBuilder {
                 for (int k = 1; k < n; ++k)
                     sets = std::max(sets, (range[k] + 1.0) / (slot(n, k) == 1 ? kPatShift1 + 1 : kPatShift2 + 1));
                 // (strict: every pattern in a set of its own)
-                const double items = strict ? chunks / kPatItem + 2 * keys.size()
+                const double items = strict ? chunks / kPatItem + 2 * nkeys
                                             : 1.3 * sets * (span / kPatItem + 1);
                 const double tab = sizeof(PatHeader) + items * sizeof(PatItem) +
-                                   (chunks / kPatItem + 2 * keys.size()) * sizeof(PatRow);
+                                   (chunks / kPatItem + 2 * nkeys) * sizeof(PatRow);
                 if ((size_t)chunks * kPatChunk * 4 > (size_t)kPatRowBytes ||
                     raw > (uint32_t)(kPatRawBytes - kPatTabBytes) || tab > kPatTabBytes - 16)
                     break;   // more channels only add to each
@@ -264,12 +293,13 @@ struct TileBuilder {
         const int nch = p->nchans;
         if (!cut(0, nch, &len, &out->cost)) return;
         // the stage being packed
-        std::vector<Item> items;
+        Items items;
         std::vector<uint32_t> trials;
         StageDesc sd{};
         uint32_t rows = 0, raw = kPatTabBytes, tab = sizeof(PatHeader);
         int groups = 0, held = 0;
         std::vector<int64_t> load(kPatFormWarps, 0);   // cost given to every forming warp so far
+        std::vector<int> order, of;                    // items by cost; the forming warp of each
         size_t last_trials = 0;                        // trial table of the last stage emitted
         auto flush_last = [&]() {
             PatTrials h;
@@ -284,17 +314,21 @@ struct TileBuilder {
             }
             held += (int)sd.nchan;
             // the costliest items first, each to the warp with the least work so far
-            std::stable_sort(items.begin(), items.end(),
-                             [](const Item& x, const Item& y) { return x.cost > y.cost; });
-            std::vector<std::vector<int>> of(kPatFormWarps);
-            std::vector<int64_t> here(kPatFormWarps, 0);
-            for (size_t i = 0; i < items.size(); ++i) {
+            const int nitems = (int)items.items.size();
+            order.resize(nitems);
+            of.resize(nitems);
+            for (int i = 0; i < nitems; ++i) order[i] = i;
+            std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+                return items.items[x].cost > items.items[y].cost;
+            });
+            int64_t here[kPatFormWarps] = {};
+            for (int i : order) {
                 int w = 0;
                 for (int v = 1; v < kPatFormWarps; ++v)
-                    if (std::make_pair(here[v], load[v]) < std::make_pair(here[w], load[w])) w = v;
-                of[w].push_back((int)i);
-                here[w] += items[i].cost;
-                load[w] += items[i].cost;
+                    if (here[v] < here[w] || (here[v] == here[w] && load[v] < load[w])) w = v;
+                of[i] = w;
+                here[w] += items.items[i].cost;
+                load[w] += items.items[i].cost;
             }
             tab = (tab + 15) & ~15u;       // copied in 16-byte pieces
             sd.addr_begin = (uint32_t)out->tab.size();
@@ -304,15 +338,16 @@ struct TileBuilder {
             out->tab.resize(out->tab.size() + (sd.addr_bytes + sd.addr_off) / 4);
             uint8_t* base = reinterpret_cast<uint8_t*>(&out->tab[sd.addr_begin]);
             PatHeader h{};
-            uint32_t n = 0, b_off = (uint32_t)(sizeof(h) + items.size() * sizeof(PatItem));
+            uint32_t n = 0, b_off = (uint32_t)(sizeof(h) + nitems * sizeof(PatItem));
             for (int w = 0; w < kPatFormWarps; ++w) {
                 h.begin[w] = (uint8_t)n;
-                for (int i : of[w]) {
-                    Item& it = items[i];
+                for (int i : order) {
+                    if (of[i] != w) continue;
+                    Item& it = items.items[i];
                     it.d.row_off = (uint16_t)b_off;
                     std::memcpy(base + sizeof(h) + n * sizeof(PatItem), &it.d, sizeof(PatItem));
-                    std::memcpy(base + b_off, it.rows.data(), it.rows.size() * sizeof(PatRow));
-                    b_off += (uint32_t)(it.rows.size() * sizeof(PatRow));
+                    std::memcpy(base + b_off, &items.rows[it.row], it.d.nrows * sizeof(PatRow));
+                    b_off += (uint32_t)(it.d.nrows * sizeof(PatRow));
                     ++n;
                 }
             }
@@ -333,7 +368,7 @@ struct TileBuilder {
         };
         Group g;
         std::vector<int> ord;
-        std::vector<Item> more;
+        Items more;
         std::vector<uint32_t> org;
         for (int c = 0; c < nch; c += len[c]) {
             make_group(c, len[c], &g);
@@ -348,24 +383,18 @@ struct TileBuilder {
                 grows += (uint32_t)(chunk_hi(q, g.u0) - chunk_lo(q, g.u0)) * kPatChunk * 4;
             for (int k = 0; k < g.n; ++k) graw += 4 * g.nwords[k];
             uint32_t chan_off[kPatMaxGroup] = {};
-            auto lay = [&]() {
-                uint32_t at = raw;
-                for (int k = 0; k < g.n; ++k) {
-                    chan_off[k] = at;
-                    at += 4 * g.nwords[k];
-                }
-                more.clear();
-                make_items(g, ord, chan_off, rows, &more, &org);
-            };
-            lay();
+            for (int k = 0; k < g.n; ++k) chan_off[k] = k > 0 ? chan_off[k - 1] + 4 * g.nwords[k - 1] : raw;
+            make_items(g, ord, chan_off, rows, &more, &org);
             if (groups > 0 && (groups == kPatStageGroups || rows + grows > (uint32_t)kPatRowBytes ||
                                raw + graw > (uint32_t)kPatRawBytes ||
-                               tab + items_bytes(more) + 15 > (uint32_t)kPatTabBytes ||
-                               items.size() + more.size() > 255)) {
+                               tab + more.bytes() + 15 > (uint32_t)kPatTabBytes ||
+                               items.items.size() + more.items.size() > 255)) {
+                const uint32_t raw_was = raw, rows_was = rows;
                 emit();
-                lay();
+                move_items(raw - raw_was, rows - rows_was, &more, &org);   // (modulo 2^32)
+                for (int k = 0; k < g.n; ++k) chan_off[k] += raw - raw_was;
             }
-            if (items_bytes(more) + tab + 15 > (uint32_t)kPatTabBytes || more.size() > 255) return;
+            if (more.bytes() + tab + 15 > (uint32_t)kPatTabBytes || more.items.size() > 255) return;
             if (groups == 0) {
                 sd = StageDesc{};
                 sd.chan_begin = (uint32_t)out->chans.size();
@@ -388,8 +417,8 @@ struct TileBuilder {
                 t[j / kPatRD * kPatPlaces + j % kPatRD] =
                     org[g.of_trial[jj]] + 4u * (uint32_t)(delay(jj, g.c) - g.u0);
             }
-            tab += items_bytes(more);
-            for (Item& it : more) items.push_back(std::move(it));
+            tab += (uint32_t)more.bytes();
+            items.append(more);
             rows += grows;
             raw += graw;
             ++groups;
@@ -439,10 +468,10 @@ double estimate_patterns(const hp_plan* p) {
         for (int i = 0; i < nd; ++i) {
             const int t = (int)((2 * i + 1) * (int64_t)ntiles / (2 * nd));
             const int d0 = pattern_tile(ndm, ntiles, t);
-            const TileBuilder b{p, d0, pattern_tile(ndm, ntiles, t + 1) - d0, false};
             for (int j = 0; j < nc; ++j) {
                 const int c = (int)((2 * j + 1) * (int64_t)p->nchans / (2 * nc)) / 8 * 8;
                 const int e = std::min(c + 8, p->nchans);
+                const TileBuilder b(p, d0, pattern_tile(ndm, ntiles, t + 1) - d0, false, c, e);
                 double cycles = 0;
                 if (!b.cut(c, e, &len, &cycles)) return -1;
                 sum += cycles / (e - c);
@@ -460,7 +489,7 @@ bool build_patterns(const hp_plan* p, DedispTiling* T) {
     try {
         std::vector<DedispTiling> parts(ntiles);
         std::vector<double> cycles(ntiles, 0.0);
-        // one thread per 1024 channels of a tile (about 1 ms)
+        // one thread per 1024 channels of a tile (about 0.5 ms)
         const int threads = (int)std::min<int64_t>((int64_t)ntiles * p->nchans / 1024, 16);
         const bool done = parallel_for(ntiles, threads, [&](int i) {
             if (failed) return;
@@ -468,7 +497,7 @@ bool build_patterns(const hp_plan* p, DedispTiling* T) {
             TileOut out;
             for (int strict = 0; strict < 2 && !out.ok; ++strict) {
                 out = TileOut();
-                TileBuilder{p, d0, d1 - d0, strict != 0}.build(&out);
+                TileBuilder(p, d0, d1 - d0, strict != 0, 0, p->nchans).build(&out);
             }
             if (!out.ok) {
                 failed = true;

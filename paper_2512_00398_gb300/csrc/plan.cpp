@@ -750,7 +750,9 @@ double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total,
 // blocks (pattern_waves) makes up for that on many short inputs: 4096 channels, 375
 // trials, 4000 samples 0.833 ms by byte rows, 0.256 by parts of pattern rows; 2048
 // channels, 200 trials, 8192 samples 0.421 and 0.160.  There the tables must earn more
-// (1.25): they cost the plan's first call 2 to 5 ms.
+// (1.25), as they make the plan's first call longer.  With both kernels' tables it takes
+// 1.2 ms more than a later one on 1024 channels x 24 trials, 3.3 on 1024 x 400, 22 on
+// 4096 x 1500 (with the byte rows' alone, built by one thread, 0.35, 3.5 and 57).
 bool patterns_pay(const hp_plan* p, double cycles, const int64_t* nout, int njobs) {
     // the default tile shape of direct dedispersion, without fused remedian levels
     if (p->dedisp_cfg != kDefaultDedispConfig || p->sb_chans > 0 || p->fuse_levels) return false;
