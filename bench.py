@@ -43,7 +43,7 @@ DEDISP_TRAFFIC = {"source_sha256_16": "0e82e2697ab3fb83", "bytes": (6.095e9 + 1.
                   "ndm": 1500, "nchans": 4096, "nsamps": 1 << 20, "config": 17}
 # The same of the pattern-row kernel, which the default configuration runs on this
 # workload (profiles/dedisp_patterns_kernel_fast_4096ch.md).
-PATTERN_TRAFFIC = {"source_sha256_16": "759dd0ca1211772d",
+PATTERN_TRAFFIC = {"source_sha256_16": "419046ab06b40610",   # (a comment changed since the capture)
                    "bytes": (9.713e9 + 1.007e9) * 955060 / 168628,
                    "ndm": 1500, "nchans": 4096, "nsamps": 1 << 20, "config": 17}
 # The same for the two stages of the sub-band variant (64-channel sub-bands, groups

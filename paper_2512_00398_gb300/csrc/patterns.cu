@@ -336,8 +336,8 @@ dedisp_patterns_kernel(const __grid_constant__ DedispBatch batch, int* status, u
         asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
         if (warp == kPatSumWarps + kPatFormWarps) {
             // Bulk copies of every stage: its set table and the channel rows' windows
-            // into a raw buffer once stage s - 3 is formed, its trial table into the slot
-            // of stage s - 5, which was summed before stage s - 3 could be formed.  A
+            // into a raw buffer once stage s - 2 is formed, its trial table into the slot
+            // of stage s - 4, which was summed before stage s - 2 could be formed.  A
             // stage's row descriptors are read a stage ahead, the stage descriptors that
             // name them two: two dependent reads from global memory take longer than a
             // stage.

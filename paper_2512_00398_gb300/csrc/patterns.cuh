@@ -46,8 +46,8 @@ struct PatTrials {
     uint32_t flush;        // 1: add the 16-bit sums to the 32-bit sums after this stage
     uint32_t pad_[2];
 };
-// Patterns of one group whose channel offsets differ by at most kPatShifts samples
-// form a set: each channel's samples are unpacked once for all of them.  Channels
+// Patterns of one group whose channel offsets differ by at most their slot's shift
+// (kPatShift1, kPatShift2) form a set: each channel's samples are unpacked once for all of them.  Channels
 // sit in four slots (of a group of three the last is empty, of two the second and
 // the last, of one the last three).  An item is 4 kPatItem words per lane of a set.
 constexpr int kPatShift1 = 1, kPatShift2 = 2;   // of slot 1; of slots 2 and 3 (slot 0: none)

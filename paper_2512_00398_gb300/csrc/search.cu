@@ -2076,7 +2076,7 @@ cudaError_t launch_walkers(const SearchArgs& a, const BaselineCtx& bc, cudaStrea
     const int64_t padding = ceil_div(n, hist_block(256)) * hist_block(256) - n;
     if (padding <= n / 8 && blocks(256) >= 300)
         hist(std::integral_constant<int, 256>{});
-    else if (blocks(64) >= 600)                           // four blocks an SM
+    else if (blocks(64) >= 600)                           // about four blocks on each of 152 SMs
         hist(std::integral_constant<int, 64>{});
     else
         hist(std::integral_constant<int, 32>{});
