@@ -28,8 +28,8 @@
 //      correctly rounded operations (ties: smallest key).
 //   4. roots are compacted in index order with a device-wide scan.
 //
-// A list of at most 1024 candidates (fewer with a large dm_tol: small_list), the usual
-// one, goes through all of it in one block's shared memory (merge_small_kernel); the
+// A list of at most 1280 candidates (fewer with friend scans or a large dm_tol: small_list),
+// the usual one, goes through all of it in one block's shared memory (merge_small_kernel); the
 // kernels of the general path then find nothing to do.  The host cannot know the count,
 // so they are launched all the same: few of them, and each starting while the one before
 // it drains.
@@ -634,32 +634,150 @@ __global__ void __launch_bounds__(kScanBlock) scatter_kernel(MergeArgs a) {
     }
 }
 
-// The whole merge of at most kSmall candidates, one per thread, in one block's shared
-// memory; it leaves *n_clamped = -1 to the general path's kernels.  Longer lists: their length,
+// The whole merge of a short list in one block's shared memory; it leaves
+// *n_clamped = -1 to the general path's kernels.  Longer lists: their length,
 // the counters, the status.  What bounds it is the chain of barriers and
 // shared-memory latencies of the sort (a list of 256 takes 3 block barriers, of
-// 1024 13) and the links.
-constexpr int kSmall = 1024;
+// 1024 13), the FP64 ratios (one each) and the links.
+constexpr int kSmall = 1280;
 
-// The longest list for one block: up to here it is faster than the general path's
-// kernels on all 152 SMs.  Links to the next dm_tol trials grow with dm_tol, and one SM
-// makes them.  One block and general path, us, lists with clusters and dense ones (those
-// of 2000 at two candidates a thread):
-//    defaults:           1024  54 and  82,  44 and 68       2000  101 and  86,   79 and  71
-//    friend scans:       1024  78 and 119, 482 and 480      2000  142 and 124, 1392 and 925
+// The longest list for one block, one candidate per thread up to 1024: up to here it is
+// not slower than the general path's kernels on all 152 SMs.  Links to the next dm_tol
+// trials grow with dm_tol, and one SM makes them; friend scans more so.  One block and
+// general path, us, lists with clusters and dense ones:
+//    defaults:           1030  71 and  89,  61 and 68       1400   90 and  83,   73 and  70
+//    friend scans:       1030  94 and 126, 513 and 535      1400  137 and 125,  861 and 667
+//    dm_tol 16:           768 140 and 132,  57 and 79       1536  345 and 151,   82 and  86
 //    dm_tol 16, scans:    512 311 and 338, 508 and 622      1024  394 and 351,  986 and 1032
+//    dm_tol 64:           256 159 and 254,  44 and 73       1024  615 and 291,   63 and  90
 //    dm_tol 64, scans:    128 377 and 321, 146 and 339       512  863 and 581,  510 and 798
-//    dm_tol 64:           128 108 and 163,  63 and 79       1024  615 and 291,  258 and 122
-int64_t small_list(int dm_tol) { return std::max(32, std::min(kSmall, 8192 / std::max(dm_tol, 1))); }
+int64_t small_list(const MergeArgs& a) {
+    const int reach = std::max(a.dm_tol, 1);
+    return std::max(32, any_window(a) ? std::min(kSmall, 16384 / reach) : std::min(1088, 8192 / reach));
+}
 
 struct SmallState {
-    uint64_t key[kSmall];
-    int64_t val[kSmall];
+    uint64_t key[2048];            // (sorted as a power of two)
+    int64_t val[2048];
     unsigned long long best[kSmall], t_lo[kSmall], t_hi[kSmall];
     int32_t parent[kSmall], rep[kSmall], members[kSmall], dm_lo[kSmall], dm_hi[kSmall];
     int32_t widths[kMaxWidths], warp_tot[32];
     uint64_t warp_max[32];
 };
+
+// Thread t holds the E entries from E t on of the list (n <= 1024 E).
+template <int E>
+__device__ __forceinline__ void merge_small(const MergeArgs& a, SmallState& s, int n) {
+    const int i0 = E * (int)threadIdx.x;
+    const int mine = min(E, n - i0);                 // entries of this thread (<= 0: none)
+    uint64_t key[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        key[e] = 0;
+        if (e < mine) {
+            const int i = i0 + e;
+            key[e] = s.key[i];
+            s.best[i] = 0;
+            s.members[i] = 0;
+            s.dm_lo[i] = INT_MAX;
+            s.dm_hi[i] = INT_MIN;
+            s.t_lo[i] = ~0ull;
+        }
+    }
+    if (any_window(a)) {
+        // components: the running maxima in t_hi, the heads in parent
+        uint64_t w[E], run = 0, total;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            w[e] = e < mine ? end_word(key[e], s.widths) : 0;
+            run = max(run, w[e]);
+        }
+        run = block_max_exclusive(run, s.warp_max, &total);
+        uint64_t h[E], last = 0;                     // head + 1 among this thread's entries
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (e < mine && (i0 + e == 0 || starts_component(key[e], run, a.t_gap)))
+                last = (uint64_t)(i0 + e + 1);
+            h[e] = last;
+            run = max(run, w[e]);
+            if (e < mine) s.t_hi[i0 + e] = run;
+        }
+        const uint64_t before = block_max_exclusive(last, s.warp_max, &total);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (e < mine) s.parent[i0 + e] = s.rep[i0 + e] = (int32_t)max(before, h[e]) - 1;
+        __syncthreads();
+        // (1024 apart: with neighbouring entries half of the threads had two and half none)
+        for (int i = threadIdx.x; i < n; i += 1024)
+            if (i + 1 == n || s.rep[i + 1] == i + 1)   // rep keeps the heads while parent changes
+                link_component(a, s.key, n, s.rep[i], i, [&](int64_t j) { return (uint64_t)s.t_hi[j]; },
+                               [&](int64_t j) { return (int64_t)s.rep[j]; }, s.parent, nullptr);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (e < mine) s.parent[i0 + e] = i0 + e;
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += 1024)
+            link_candidate(a, s.widths, s.key, n, i, s.parent, nullptr);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (e < mine) {
+            s.rep[i0 + e] = INT_MAX;
+            s.t_hi[i0 + e] = 0;
+        }
+    __syncthreads();
+    double snr[E];
+    int32_t root[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        if (e >= mine) continue;
+        const uint64_t k = key[e];
+        const int32_t r = root[e] = uf_find(s.parent, i0 + e);
+        s.parent[i0 + e] = r;
+        snr[e] = cand_snr(a, s.widths, k, s.val[i0 + e]);
+        atomicMax(&s.best[r], (unsigned long long)__double_as_longlong(snr[e]));
+        atomicAdd(&s.members[r], 1);
+        atomicMin(&s.dm_lo[r], key_dm(k));
+        atomicMax(&s.dm_hi[r], key_dm(k));
+        const unsigned long long ts = (unsigned long long)key_sample(k);
+        atomicMin(&s.t_lo[r], ts);
+        atomicMax(&s.t_hi[r], ts + (unsigned long long)s.widths[key_width(k)]);
+    }
+    __syncthreads();
+    int32_t roots = 0, total;
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (e < mine) {
+            if ((unsigned long long)__double_as_longlong(snr[e]) == s.best[root[e]])
+                atomicMin(&s.rep[root[e]], i0 + e);
+            roots += root[e] == i0 + e;
+        }
+    int64_t slot = block_exclusive(roots, s.warp_tot, &total);   // (synchronises)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = i0 + e;
+        if (e >= mine || root[e] != i) continue;
+        if (slot < a.out_cap) {
+            const int32_t rp = s.rep[i];
+            const uint64_t kr = s.key[rp];
+            hp_cand c;
+            c.dm_idx = key_dm(kr);
+            c.width_idx = key_width(kr);
+            c.sample = key_sample(kr);
+            c.snr = (float)cand_snr(a, s.widths, kr, s.val[rp]);
+            c.members = s.members[i];
+            c.dm_lo = s.dm_lo[i];
+            c.dm_hi = s.dm_hi[i];
+            c.t_lo = (int64_t)s.t_lo[i];
+            c.t_hi = (int64_t)s.t_hi[i];
+            a.out[slot] = c;
+        }
+        ++slot;
+    }
+    if (threadIdx.x == 0) *a.out_count = total;
+}
 
 __global__ void __launch_bounds__(1024) merge_small_kernel(MergeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -678,88 +796,23 @@ __global__ void __launch_bounds__(1024) merge_small_kernel(MergeArgs a) {
     const int n = nc > 0 ? (int)nc : 0;
     int size = 64;
     while (size < n) size <<= 1;
-    if (t < size) {
-        s.key[t] = kPad;
-        s.val[t] = 0;
-        if (t < n) {
-            const hp_raw_cand c = a.raw[t];
-            s.key[t] = cand_key(c);
-            s.val[t] = c.S;
+    for (int i = t; i < size; i += 1024) {
+        s.key[i] = kPad;
+        s.val[i] = 0;
+        if (i < n) {
+            const hp_raw_cand c = a.raw[i];
+            s.key[i] = cand_key(c);
+            s.val[i] = c.S;
         }
-        s.best[t] = 0;
-        s.members[t] = 0;
-        s.dm_lo[t] = INT_MAX;
-        s.dm_hi[t] = INT_MIN;
-        s.t_lo[t] = ~0ull;
     }
     if (t < a.nw) s.widths[t] = a.widths[t];
     __syncthreads();
     bitonic_sort(s.key, s.val, size);
     __syncthreads();
-    if (any_window(a)) {
-        // components: the running maxima in t_hi, the heads in parent
-        const uint64_t key = t < n ? s.key[t] : 0;
-        const uint64_t w = t < n ? end_word(key, s.widths) : 0;
-        uint64_t total;
-        const uint64_t before = block_max_exclusive(w, s.warp_max, &total);
-        const bool head = t < n && (t == 0 || starts_component(key, before, a.t_gap));
-        const uint64_t mine = head ? t + 1 : 0;
-        const uint64_t h = max(mine, block_max_exclusive(mine, s.warp_max, &total));
-        if (t < n) {
-            s.t_hi[t] = max(before, w);
-            s.parent[t] = s.rep[t] = (int32_t)h - 1;
-        }
-        __syncthreads();
-        if (t < n && (t + 1 == n || s.rep[t + 1] == t + 1))   // rep keeps the heads while parent changes
-            link_component(a, s.key, n, s.rep[t], t, [&](int64_t j) { return (uint64_t)s.t_hi[j]; },
-                           [&](int64_t j) { return (int64_t)s.rep[j]; }, s.parent, nullptr);
-    } else {
-        if (t < n) s.parent[t] = t;
-        __syncthreads();
-        if (t < n) link_candidate(a, s.widths, s.key, n, t, s.parent, nullptr);
-    }
-    __syncthreads();
-    if (t < n) {
-        s.rep[t] = INT_MAX;
-        s.t_hi[t] = 0;
-    }
-    __syncthreads();
-    const uint64_t k = t < n ? s.key[t] : 0;
-    const double snr = t < n ? cand_snr(a, s.widths, k, s.val[t]) : 0.0;
-    int32_t r = 0;
-    if (t < n) {
-        r = uf_find(s.parent, t);
-        s.parent[t] = r;
-        atomicMax(&s.best[r], (unsigned long long)__double_as_longlong(snr));
-        atomicAdd(&s.members[r], 1);
-        atomicMin(&s.dm_lo[r], key_dm(k));
-        atomicMax(&s.dm_hi[r], key_dm(k));
-        const unsigned long long ts = (unsigned long long)key_sample(k);
-        atomicMin(&s.t_lo[r], ts);
-        atomicMax(&s.t_hi[r], ts + (unsigned long long)s.widths[key_width(k)]);
-    }
-    __syncthreads();
-    if (t < n && (unsigned long long)__double_as_longlong(snr) == s.best[r]) atomicMin(&s.rep[r], t);
-    __syncthreads();
-    const bool root = t < n && r == t;
-    int32_t total;
-    const int64_t slot = block_exclusive(root, s.warp_tot, &total);
-    if (root && slot < a.out_cap) {
-        const int32_t rp = s.rep[t];
-        const uint64_t kr = s.key[rp];
-        hp_cand c;
-        c.dm_idx = key_dm(kr);
-        c.width_idx = key_width(kr);
-        c.sample = key_sample(kr);
-        c.snr = (float)cand_snr(a, s.widths, kr, s.val[rp]);
-        c.members = s.members[t];
-        c.dm_lo = s.dm_lo[t];
-        c.dm_hi = s.dm_hi[t];
-        c.t_lo = (int64_t)s.t_lo[t];
-        c.t_hi = (int64_t)s.t_hi[t];
-        a.out[slot] = c;
-    }
-    if (t == 0) *a.out_count = total;
+    if (n <= 1024)
+        merge_small<1>(a, s, n);
+    else
+        merge_small<2>(a, s, n);
 }
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
@@ -792,7 +845,7 @@ std::atomic<int> g_wave[11];
 
 cudaError_t launch_merge(const MergeArgs& a_in, cudaStream_t s, int64_t* nlaunch) {
     MergeArgs a = a_in;
-    a.small_max = small_list(a.dm_tol);
+    a.small_max = small_list(a);
     if (a.cap <= 0) {
         return cudaMemsetAsync(a.out_count, 0, sizeof(int64_t), s);
     }

@@ -1,6 +1,7 @@
-"""The list lengths at which the merge leaves its one block for the whole GPU (1024
-candidates, fewer with many trials in reach), against the oracle; and a dense list whose
-friend scans one block would make alone."""
+"""The list lengths at which the merge leaves its one block for the whole GPU (1280
+candidates, 1088 with friend scans, fewer with many trials in reach) and takes two
+candidates a thread (1025), against the oracle; and a dense list whose friend scans one
+block would make alone."""
 import numpy as np
 import pytest
 
@@ -36,12 +37,13 @@ def _plan(hp, widths, **kw):
                    raw_capacity=65536, **kw)
 
 
-# (min(1024, 8192 / dm_tol), at least 32; any width a friend's, or friend scans)
-@pytest.mark.parametrize("w_tol", [13, 1])
-@pytest.mark.parametrize("dm_tol,limit", [(0, 1024), (1, 1024), (9, 910), (70, 117), (399, 32)])
-def test_around_the_limit(env, dm_tol, limit, w_tol):
+# (any width a friend's, or friend scans)
+@pytest.mark.parametrize("dm_tol,w_tol,limit", [
+    (0, 13, 1280), (1, 13, 1280), (1, 13, 1024), (16, 13, 1024), (70, 13, 234), (399, 13, 41),
+    (0, 1, 1088), (1, 1, 1088), (1, 1, 1024), (9, 1, 910), (70, 1, 117), (399, 1, 32)])
+def test_around_the_limit(env, dm_tol, w_tol, limit):
     torch, hp, widths = env
-    recs, sigma = raw_list(31, 1200, ndm=NDM, nout=NOUT, nw=13, members=(5, 60), dm_spread=3, t_spread=60)
+    recs, sigma = raw_list(31, 1500, ndm=NDM, nout=NOUT, nw=13, members=(5, 60), dm_spread=3, t_spread=60)
     with _plan(hp, widths, dm_tol=dm_tol, w_tol=w_tol) as p:
         for n in (limit - 1, limit, limit + 1):
             raw, cnt, sig = _upload(torch, hp, recs[:n], sigma)
