@@ -6,7 +6,7 @@
  *   incoherent dedispersion over every trial DM  ->  per trial: baseline
  *   removal, normalisation, boxcar matched filtering, peak detection  ->
  *   candidate merging / clustering in (DM, time, width).
- * RFI mitigation (first GPU stage of Algorithm 1) is not part of this path.
+ * RFI mitigation (first GPU stage of Algorithm 1) is an option (HP_PARAM_RFI).
  *
  * Conventions shared by every call:
  *   - Return value: HP_OK (0) or a negative HP_ERR_* code.  Argument errors are
@@ -203,9 +203,8 @@ int hp_plan_workspace_bytes(const hp_plan* plan, int64_t nsamps, size_t* bytes);
 
 /* Give the plan a caller-owned device workspace (256-byte aligned, at least
  * hp_plan_workspace_bytes).  While bound, the plan allocates no scratch, only
- * its constant tables (hp_plan_prepare); the
- * caller keeps ownership and must keep it alive until the plan is destroyed
- * or another workspace is bound.  Passing NULL unbinds (the plan then
+ * its constant tables (hp_plan_prepare); the caller keeps ownership and must
+ * keep it alive until the plan is destroyed or another workspace is bound.  Passing NULL unbinds (the plan then
  * allocates its own scratch with cudaMalloc on demand, grow-only).  The size
  * depends on the raw capacity and baseline mode: query it after setting them. */
 int hp_plan_bind_workspace(hp_plan* plan, void* workspace_dev, size_t bytes);
@@ -216,8 +215,9 @@ int hp_plan_bind_workspace(hp_plan* plan, void* workspace_dev, size_t bytes);
  * tables.  There are two of these, each up to tens of MB (4096 channels, 1500 trials):
  * those of the tile shape, built by the plan's first call, and with the default shape
  * those of the pattern rows, built by the first call, which may be a later one, whose
- * length makes them pay, and kept for every call after it.  Without them, while `stream` is captured
- * and where their allocation is refused, the byte rows run instead (same sums).
+ * length makes them pay, and kept for every call after it.  Without them, as in a call
+ * that is captured before they are built or where their allocation is refused, the byte
+ * rows run instead (same sums).
  * Waits for `stream`; HP_ERR_NSAMPS_TOO_SHORT as for hp_search. */
 int hp_plan_prepare(hp_plan* plan, int64_t nsamps, void* stream);
 
@@ -304,9 +304,9 @@ int hp_plan_autotune(hp_plan* plan, const uint8_t* filterbank_dev, int64_t nsamp
 /* ------------------------------------------------------------ batching */
 /* Many filterbanks of uneven length, channel count and sampling time searched
  * together -- the multi-file workload that the paper (Section IV-C) serves
- * with a two-stage pipeline of CPU threads and task queues.  Here every file's
- * dedispersion tiles go into ONE kernel launch, the per-file search and merge
- * chains run side by side on internal streams, and the whole sequence is
+ * with a two-stage pipeline of CPU threads and task queues.  Here the files are
+ * dedispersed one after another, largest first, each file's search and merge
+ * run beside the next ones' dedispersion on internal streams, and the whole sequence is
  * captured once into a CUDA graph and replayed while the inputs, sizes and
  * outputs stay the same.  Results are identical to hp_search per file.
  *   plans  host array of nfiles (1..HP_BATCH_MAX_FILES) caller-owned plans, one

@@ -1297,8 +1297,6 @@ int batch_dedisp(hp_batch* b, int i, const Layout& L, uint8_t* ws, bool fuse, cu
     return rc;
 }
 
-// Enqueue the whole batch on s: one transpose launch, one dedispersion launch
-// over every file's tiles, then per file search + merge on a side stream.
 // One call of a batch: one transpose launch over every file; then the files'
 // dedispersion launches one after another on the caller's stream, largest
 // first, and each file's search and merge on its own side stream as soon as
