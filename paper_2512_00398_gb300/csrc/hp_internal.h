@@ -82,6 +82,12 @@ struct TileDesc {
 };
 
 // Host copy of the tiling of one plan for one config.
+// Estimated SM cycles of the pattern-row kernel per time tile: summed over the DM tiles,
+// and of the costliest of them.
+struct PatternCost {
+    double sum = 0, top = 0;
+};
+
 struct DedispTiling {
     int cfg = -1;
     int BD = 0, BT = 0;
@@ -90,8 +96,8 @@ struct DedispTiling {
     std::vector<ChanDesc> chans;
     std::vector<uint32_t> addr;    // per stage [pair][BD][2] byte offsets in the stage buffer
                                    // (pattern rows: the stage tables of patterns.cuh)
-    bool pattern = false;          // tables of the pattern-row kernel (patterns.cu), with its
-    double cycles = 0;             // estimated SM cycles per time tile, summed over the DM tiles
+    bool pattern = false;          // tables of the pattern-row kernel (patterns.cu), which cost this
+    PatternCost cost;
     int64_t max_reach = 0;         // max over rows of goff + row bytes
 };
 

@@ -68,11 +68,16 @@ struct TileBuilder {
     const int32_t* delays(int c) const { return &column[(size_t)(c - col0) * nd]; }
     int32_t delay(int j, int c) const { return delays(c)[j]; }
 
-    // Estimated SM cycles of a group whose sets unpack `sets` chunks in all and put
-    // `rows` chunks into rows; fitted to 1620 cycles per group (15 and 51 chunks) at
-    // 4096 channels, 1700 (16, 56) at 2048 and 2320 (26, 88) at 1024, 24 trials each.
+    // Cost of a group whose sets unpack `sets` chunks in all and put `rows` chunks into
+    // rows, by which the channels are cut into groups (about SM cycles: 1620 per group of
+    // 15 and 51 chunks at 4096 channels, 24 trials).
     double group_cost(double sets, double rows) const {
         return 150.0 + 21.0 * nd + 21.0 * sets + 13.0 * rows;
+    }
+    // Its SM cycles, fitted to the 3645 whole-tile launches of plan.cpp (pattern_cycles) that
+    // have one wave or tiles alike: measured / estimated 0.97-1.04 (5th to 95th of 100).
+    double group_cycles(double sets, double rows) const {
+        return 636.0 + 8.7 * nd + 19.5 * sets + 10.6 * rows;
     }
 
     void make_group(int c, int n, Group* g) const {
@@ -219,9 +224,10 @@ struct TileBuilder {
         for (uint32_t& o : *org) o += row;
     }
 
-    // The cheapest cut of the channels [begin, nch) into groups of 1 .. kPatMaxGroup.
+    // The cheapest cut of the channels [begin, nch) into groups of 1 .. kPatMaxGroup;
+    // total: its SM cycles.
     bool cut(int begin, int nch, std::vector<uint8_t>* len, double* total) const {
-        std::vector<double> best(nch + 1, 0.0);
+        std::vector<double> best(nch + 1, 0.0), cycles(nch + 1, 0.0);
         len->assign(nch, 0);
         int cls[kPatBD];
         uint64_t keys[kPatBD];             // the patterns, by refinement: class, relative delay
@@ -279,12 +285,13 @@ struct TileBuilder {
                 const double cost = group_cost(sets * (span + 1), chunks) + best[c + n];
                 if (cost < best[c]) {
                     best[c] = cost;
+                    cycles[c] = group_cycles(sets * (span + 1), chunks) + cycles[c + n];
                     (*len)[c] = (uint8_t)n;
                 }
             }
             if ((*len)[c] == 0) return false;
         }
-        *total = best[begin];
+        *total = cycles[begin];
         return true;
     }
 
@@ -452,35 +459,42 @@ bool parallel_for(int n, int threads, const std::function<void(int)>& f) {
     return !failed;
 }
 
-// 83 sums per SM and cycle (1.61 M cycles per block of 15 trials x 2176 samples on
-// the 4096-channel file; 82 at 1024 channels).
-double byte_row_cycles(double sums) { return sums / 83.0; }
+// (the launches of plan.cpp, pattern_cycles: measured / estimated 0.99-1.02, 5th to 95th of 100)
+double byte_row_cycles(double sums) { return sums / 79.0; }
 
 // First trial of DM tile i.
 static int pattern_tile(int ndm, int ntiles, int i) { return (int)((int64_t)ndm * i / ntiles); }
 
-double estimate_patterns(const hp_plan* p) {
+PatternCost estimate_patterns(const hp_plan* p) {
     const int ndm = p->ndm(), ntiles = (ndm + kPatBD - 1) / kPatBD;
-    const int nd = std::min(ntiles, 3), nc = std::min(p->nchans / 8 + 1, 8);
-    double sum = 0;
+    const int nd = std::min(ntiles, 5), nc = std::min(p->nchans / 8 + 1, 8);
+    PatternCost cost;
+    int last = 0;                     // the tile before, and its cycles: straight lines between
+    double before = 0;
     std::vector<uint8_t> len;
     try {
         for (int i = 0; i < nd; ++i) {
-            const int t = (int)((2 * i + 1) * (int64_t)ntiles / (2 * nd));
+            const int t = nd > 1 ? (int)((int64_t)i * (ntiles - 1) / (nd - 1)) : 0;
             const int d0 = pattern_tile(ndm, ntiles, t);
+            double tile = 0;
             for (int j = 0; j < nc; ++j) {
                 const int c = (int)((2 * j + 1) * (int64_t)p->nchans / (2 * nc)) / 8 * 8;
                 const int e = std::min(c + 8, p->nchans);
                 const TileBuilder b(p, d0, pattern_tile(ndm, ntiles, t + 1) - d0, false, c, e);
                 double cycles = 0;
-                if (!b.cut(c, e, &len, &cycles)) return -1;
-                sum += cycles / (e - c);
+                if (!b.cut(c, e, &len, &cycles)) return PatternCost{-1, 0};
+                // (eight channels alone make 1.5% more of them than a whole tile's cut)
+                tile += cycles / (e - c) / nc * p->nchans / 1.015;
             }
+            cost.sum += tile + (t - last > 1 ? 0.5 * (t - last - 1) * (before + tile) : 0.0);
+            cost.top = std::max(cost.top, tile);
+            last = t;
+            before = tile;
         }
     } catch (...) {
-        return -1;
+        return PatternCost{-1, 0};
     }
-    return sum / (nd * nc) * p->nchans * ntiles;
+    return cost;
 }
 
 bool build_patterns(const hp_plan* p, DedispTiling* T) {
@@ -513,7 +527,10 @@ bool build_patterns(const hp_plan* p, DedispTiling* T) {
         });
         if (!done || failed) return false;
         append_tiling(parts, T);
-        for (double c : cycles) T->cycles += c;
+        for (double c : cycles) {
+            T->cost.sum += c;
+            T->cost.top = std::max(T->cost.top, c);
+        }
     } catch (...) {
         *T = DedispTiling();
         return false;

@@ -704,26 +704,24 @@ bool reach_ok(const hp_plan* p, int64_t nout, int64_t xt_pitch) {
     return last_t0 + p->tiling.max_reach <= xt_pitch;
 }
 
-// Waves of `total` pattern-row blocks, in units of a whole tile's time, if the tiles of
-// the last *cols of the last input's ntt time columns (0: none) are shared by *parts
-// blocks each.  A block takes a tile's channels one after another for up to a
-// millisecond, and one block fits an SM: 320 blocks (375 trials, four gulps) on 152 SMs
-// took three such waves where 2.1 would do.  A part takes 1 / parts of a wave and
+// How a launch of `total` pattern-row blocks is divided: the tiles of the last *cols of the
+// last input's ntt time columns (0: none) are shared by *parts blocks each, where that
+// takes the fewest waves, of tiles alike.  A block takes a tile's channels one after
+// another for up to a millisecond, and one block fits an SM: 320 blocks (375 trials, four
+// gulps) on 152 SMs took three such waves where 2.1 would do.  A part takes 1 / parts of a wave and
 // `fixed` more to fill its pipeline and to add its sums to the output; a
 // gain of less than 4% or 0.15 waves is left, as the kernel that takes parts of tiles is
 // 1 to 2% slower and tiles of high delays take longer than the others.  Measured, whole
 // tiles and parts by this rule, 4096 channels: 1500 trials x 9215 samples (2.07 waves)
 // 2.12 and 1.58 ms; 375 x 83968 (4.32) 4.06 and 3.64; 1500 x 129 000 (26.1) 12.80 and
 // 12.61; 750 x 8192 (0.84) 0.833, 0.869 split against the rule.
-double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total, int ntt, int* cols,
-                     int* parts) {
+void pattern_waves(const hp_plan* p, const PatternCost& cost, int64_t total, int ntt, int* cols, int* parts) {
     *cols = 0;
     *parts = 1;
-    const int64_t sms = p->sm_count;
-    double best = (double)ceil_div(total, sms);
-    if (nq <= 0 || cycles <= 0) return best;
+    const int64_t sms = p->sm_count, nq = ceil_div(p->ndm(), kPatBD);
+    const double best = (double)ceil_div(total, sms);
     double limit = best - std::max(0.04 * best, 0.15);
-    const double fixed = 20000.0 * (double)nq / cycles;
+    const double fixed = 20000.0 * (double)nq / cost.sum;
     const int max_parts = std::min(16, p->nchans / 64);
     for (int c = 1; c <= std::min(ntt, 24) && c * nq <= 2 * sms; ++c)
         for (int k = 2; k <= max_parts; ++k) {
@@ -733,45 +731,73 @@ double pattern_waves(const hp_plan* p, double cycles, int64_t nq, int64_t total,
             const int64_t rest = c * nq * k - (waves * sms - whole) * (int64_t)(1.0 / unit);
             const double t = (double)waves + (rest > 0 ? (double)ceil_div(rest, sms) * unit : 0.0);
             if (t < limit) {
-                best = limit = t;
+                limit = t;
                 *cols = c;
                 *parts = k;
             }
         }
-    return best;
 }
 
-// Is a launch of njobs inputs (nout[j] samples) faster with pattern rows that take
-// `cycles` per time tile?  Both kernels keep one block per SM, so the one whose last
-// wave ends first, by the estimated cycles of its blocks: the pattern rows' larger
-// tiles (24 trials x 2048 samples against 15 x 2176) lose on short inputs, where a
-// wave is nearly empty, although they take fewer cycles per sum.  (The 1.03 leaves
-// near ties, within the estimates' error, to the byte rows.)  Sharing tiles among
-// blocks (pattern_waves) makes up for that on many short inputs: 4096 channels, 375
+// To start a block and fill and drain its pipeline, from a launch's second wave on (either
+// kernel; the first is part of every launch).
+constexpr double kBlockCycles = 12000.0;
+
+// Estimated SM cycles of a launch so divided.  Tiles of high delays have more patterns, up
+// to ten times the cycles of the first ones on a grid that widens with the DM, and come
+// last: a launch ends with some of those, whatever the average.  Zeroing the output for
+// the parts is a launch more.  Fitted, as the other estimates here, to 4837 launches
+// (100-4096 channels, 20-1500 trials, 1000-150 000 samples, even and widening grids) and
+// 20 555 divisions of them: measured / estimated 0.96-1.03 for whole tiles and 0.93-1.10
+// for parts (5th to 95th of 100; no better with the blocks' order simulated).
+double pattern_cycles(const hp_plan* p, const PatternCost& cost, int64_t total, int cols, int parts) {
+    const double sms = p->sm_count, nq = (double)ceil_div(p->ndm(), kPatBD);
+    auto waves = [&](double n, double each, double last) {
+        const double w = std::ceil(n / sms);
+        return w <= 1 ? last : std::max(w * each, std::min((w - 1) * each + last, n * each / sms + 0.7 * last));
+    };
+    const double tile = cost.sum / nq + kBlockCycles, last = cost.top + kBlockCycles;
+    if (cols == 0) return waves((double)total, tile, last) - kBlockCycles;
+    const double n = cols * nq * parts, whole = (double)total - cols * nq;
+    const double part = 1.04 * cost.sum / nq / parts + 28000.0, end = 1.04 * cost.top / parts + 28000.0;
+    // (the parts fill SMs from the last whole wave on)
+    return 10000.0 + (whole <= 0 ? waves(n, part, end)
+                                 : std::max(1.02 * waves(whole, tile, last),
+                                            (1.02 * whole * tile + n * part) / sms + 0.7 * end));
+}
+
+// Is a launch of njobs inputs (nout[j] samples) faster with pattern rows of tiles that
+// cost that much?  Both kernels keep one block per SM, so the one whose last wave ends first,
+// by the estimated cycles of its blocks: the pattern rows' larger tiles (24 trials x 2048
+// samples against 15 x 2176) lose on short inputs, where a wave is nearly empty, and
+// where the last tiles share little, although they take fewer cycles per sum; sharing
+// tiles among blocks (pattern_waves) makes up for that on many short inputs: 4096 channels, 375
 // trials, 4000 samples 0.833 ms by byte rows, 0.256 by parts of pattern rows; 2048
-// channels, 200 trials, 8192 samples 0.421 and 0.160.  There the tables must earn more
-// (1.25), as they make the plan's first call longer.  With both kernels' tables it takes
+// channels, 200 trials, 8192 samples 0.421 and 0.160.  (Near ties of parts, whose
+// estimate is the rougher one, go to the byte rows, those of whole tiles to the pattern
+// rows: these lose less beside other files' searches -- a batch of four files with one
+// such tie 18.44 and 18.71 ms.)  On 2500 launches like those above, but others, this takes
+// 0.60 of the byte rows' time (geometric mean), and 11 are more than 3% slower than byte
+// rows, up to 1.2 times (256 channels, parts); by the average tile they were 102, up to 2.2
+// times (512 channels, 240 trials to DM 312, 8000 samples: 0.194 and 0.123 ms).  The tables make the plan's first call longer: with both kernels' it takes
 // 1.2 ms more than a later one on 1024 channels x 24 trials, 3.3 on 1024 x 400, 22 on
 // 4096 x 1500 (with the byte rows' alone, built by one thread, 0.35, 3.5 and 57).
-bool patterns_pay(const hp_plan* p, double cycles, const int64_t* nout, int njobs) {
+bool patterns_pay(const hp_plan* p, const PatternCost& cost, const int64_t* nout, int njobs) {
     // the default tile shape of direct dedispersion, without fused remedian levels
     if (p->dedisp_cfg != kDefaultDedispConfig || p->sb_chans > 0 || p->fuse_levels) return false;
-    if (cycles <= 0 || njobs < 1) return false;
+    if (cost.sum <= 0 || njobs < 1) return false;
     const DedispTiling& T = p->tiling;
-    const int64_t nt = (int64_t)T.tiles.size(), nq = ceil_div(p->ndm(), kPatBD);
     int64_t qcols = 0, tcols = 0;
     for (int j = 0; j < njobs; ++j) {
         if (nout[j] <= 0) return false;
         qcols += ceil_div(nout[j], kPatBT);
         tcols += ceil_div(nout[j], T.BT);
     }
-    const double tile = cycles / (double)nq;
-    const double q = (double)ceil_div(qcols * nq, p->sm_count) * tile;
-    const double t = (double)ceil_div(tcols * nt, p->sm_count) *
-                     byte_row_cycles((double)T.BD * p->nchans * T.BT);
+    const double t = (double)ceil_div(tcols * (int64_t)T.tiles.size(), p->sm_count) *
+                     (byte_row_cycles((double)T.BD * p->nchans * T.BT) + kBlockCycles) - kBlockCycles;
+    const int64_t total = qcols * ceil_div(p->ndm(), kPatBD);
     int cols, parts;
-    return q * 1.03 < t || pattern_waves(p, cycles, nq, qcols * nq, (int)ceil_div(nout[njobs - 1], kPatBT),
-                                         &cols, &parts) * tile * 1.25 < t;
+    pattern_waves(p, cost, total, (int)ceil_div(nout[njobs - 1], kPatBT), &cols, &parts);
+    return pattern_cycles(p, cost, total, cols, parts) * (cols > 0 ? 1.03 : 0.98) < t;
 }
 
 bool use_patterns(const hp_plan* p, const int64_t* nout, const int64_t* xt_pitch, int njobs) {
@@ -779,7 +805,7 @@ bool use_patterns(const hp_plan* p, const int64_t* nout, const int64_t* xt_pitch
     if (!p->ptables) return false;
     for (int j = 0; j < njobs; ++j)
         if ((ceil_div(nout[j], Q.BT) - 1) * Q.BT + Q.max_reach > xt_pitch[j]) return false;
-    return patterns_pay(p, Q.cycles, nout, njobs);
+    return patterns_pay(p, Q.cost, nout, njobs);
 }
 
 // While it lives, this thread's allocations and copies are allowed beside another
@@ -792,10 +818,16 @@ struct BesideCaptures {
 };
 
 int prepare_patterns(hp_plan* p, int64_t nout, int njobs, cudaStream_t s) {
-    if (p->ptables || p->pat_estimate < 0 || p->dedisp_cfg != kDefaultDedispConfig ||
+    if (p->ptables || p->pat_estimate.sum < 0 || p->dedisp_cfg != kDefaultDedispConfig ||
         p->sb_chans > 0 || p->fuse_levels)
         return HP_OK;
-    if (p->pat_estimate == 0) p->pat_estimate = estimate_patterns(p);
+    if (p->pat_estimate.sum == 0) {
+        // (of 1250 plans 98 in 100 come out 4% above to 5% below their tables' own cost: a
+        // near tie builds them and is decided by that)
+        p->pat_estimate = estimate_patterns(p);
+        p->pat_estimate.sum *= 0.96;
+        p->pat_estimate.top *= 0.96;
+    }
     int64_t nouts[kMaxJobs];
     std::fill_n(nouts, kMaxJobs, nout);
     if (!patterns_pay(p, p->pat_estimate, nouts, std::min(njobs, kMaxJobs))) return HP_OK;
@@ -804,7 +836,7 @@ int prepare_patterns(hp_plan* p, int64_t nout, int njobs, cudaStream_t s) {
         return HP_OK;
     DedispTiling& Q = p->ptiling;
     if (!Q.pattern && !build_patterns(p, &Q)) {
-        p->pat_estimate = -1;
+        p->pat_estimate.sum = -1;
         return HP_OK;
     }
     size_t off = 0;
@@ -822,7 +854,7 @@ int prepare_patterns(hp_plan* p, int64_t nout, int njobs, cudaStream_t s) {
     int rc = plan_alloc(p, off, &mem);
     if (rc) {               // no room: the byte rows run, from now on (no call asks again)
         Q = DedispTiling();
-        p->pat_estimate = -1;
+        p->pat_estimate.sum = -1;
         return HP_OK;
     }
     uint8_t* b = (uint8_t*)mem;
@@ -855,7 +887,7 @@ void drop_patterns(hp_plan* p) {
     p->ptables = nullptr;
     p->ptables_bytes = 0;
     p->ptiling = DedispTiling();
-    p->pat_estimate = -1;
+    p->pat_estimate.sum = -1;
 }
 
 DedispJob make_job(const hp_plan* p, const uint8_t* xt, int64_t xt_pitch, int32_t* out,
@@ -889,7 +921,7 @@ int split_tail(const hp_plan* p, DedispBatch* b, cudaStream_t s) {
     DedispJob& J = b->jobs[b->njobs - 1];
     const int64_t nq = J.ndt;
     int cols = 0, parts = 1;
-    pattern_waves(p, p->ptiling.cycles, nq, b->prefix[b->njobs], J.ntt, &cols, &parts);
+    pattern_waves(p, p->ptiling.cost, b->prefix[b->njobs], J.ntt, &cols, &parts);
     if (cols == 0) return HP_OK;
     DedispJob& Q = b->jobs[b->njobs];
     Q = J;
@@ -1635,7 +1667,7 @@ int hp_plan_set_allocator(hp_plan* p, hp_alloc_fn alloc, hp_free_fn free_fn, voi
         p->ws_own_bytes = 0;
         if (st != 0) p->pending_status = st;
     }
-    if (!p->ptables) p->pat_estimate = 0;   // the new allocator may have room for the tables
+    if (!p->ptables) p->pat_estimate = PatternCost();   // the new allocator may have room for the tables
     p->alloc_fn = alloc;
     p->free_fn = free_fn;
     p->alloc_ctx = ctx;

@@ -85,8 +85,8 @@ struct hp_plan {
     // Pattern-row tables, beside those of the default tile shape: built by the first
     // input that the pattern-row kernel is estimated to be faster on.
     hp::DedispTiling ptiling;
-    double pat_estimate = 0;           // SM cycles per time tile, all DM tiles, from a few of them
-                                       // (0: not estimated yet, < 0: no tables can be laid out or held)
+    hp::PatternCost pat_estimate;      // from a few tiles and channels (sum 0: not estimated yet,
+                                       // < 0: no tables can be laid out or held)
     void* ptables = nullptr;
     size_t ptables_bytes = 0;
     int sm_count = 148;
@@ -150,9 +150,9 @@ int ensure_workspace(hp_plan* p, size_t need, uint8_t** base);
 // Tables of the pattern-row kernel for the plan's direct delays; false (T left
 // empty) where they cannot be laid out.
 bool build_patterns(const hp_plan* p, DedispTiling* T);
-// Its SM cycles per time tile, summed over the DM tiles, from a sample of the tiles
-// and channels; < 0 where a channel cannot be laid out.
-double estimate_patterns(const hp_plan* p);
+// Their cost from a sample of the tiles and channels; sum < 0 where a channel cannot
+// be laid out.
+PatternCost estimate_patterns(const hp_plan* p);
 // Build the pattern-row tables if a launch of njobs inputs of nout samples is
 // estimated to be faster with them and s is not being captured (nothing can be
 // allocated then; the byte rows run).
@@ -166,7 +166,8 @@ int launched_kernel(const DedispBatch& b);
 void drop_patterns(hp_plan* p);
 // Append the tiles of every part, whose indices count from its own tables (left empty).
 void append_tiling(std::vector<DedispTiling>& parts, DedispTiling* T);
-// Estimated SM cycles of the byte-row kernel for `sums` (trial, channel, sample) sums.
+// Estimated SM cycles of a block of the byte-row kernel with so many (trial, channel,
+// sample) sums.
 double byte_row_cycles(double sums);
 // f(i) for i in [0, n) on up to `threads` host threads; false if one threw.
 bool parallel_for(int n, int threads, const std::function<void(int)>& f);

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 def test_tables_built_beside_a_capture(hp):                           # noqa: F811
     import torch
     nchans, nout = 96, 60 * 2048 + 9        # (3000 samples: byte rows)
-    dms = np.linspace(0.0, 200.0, 48).astype(np.float32)
+    dms = np.linspace(0.0, 600.0, 48).astype(np.float32)
     delays = oracle.delays(nchans, 1500.0, BW, TSAMP, dms)
     rng = np.random.Generator(np.random.PCG64(23))
     x = rng.integers(0, 256, size=(nout + int(delays.max()), nchans), dtype=np.uint8)

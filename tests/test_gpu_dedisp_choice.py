@@ -43,7 +43,7 @@ def test_shared_tiles(hp, shape):                                     # noqa: F8
 
 # (unlike trials; a single wave of byte rows)
 @pytest.mark.parametrize("nchans,bw,ndm,hi,nout", [(128, -1.953125, 100, 400, 70001),
-                                                   (96, BW, 48, 200, 3001)])
+                                                   (96, BW, 48, 600, 3001)])
 def test_byte_rows_kept(hp, nchans, bw, ndm, hi, nout):               # noqa: F811
     import torch
     from paper_2512_00398_gb300 import synth

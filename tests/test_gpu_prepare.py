@@ -13,7 +13,7 @@ NCHANS, NOUT = 96, 60 * 2048 + 9            # (3000 samples: byte rows)
 
 @pytest.fixture(scope="module")
 def case():
-    dms = np.linspace(0.0, 200.0, 48).astype(np.float32)
+    dms = np.linspace(0.0, 600.0, 48).astype(np.float32)
     delays = oracle.delays(NCHANS, 1500.0, BW, TSAMP, dms)
     rng = np.random.Generator(np.random.PCG64(41))
     x = rng.integers(0, 256, size=(NOUT + int(delays.max()), NCHANS), dtype=np.uint8)
